@@ -493,12 +493,6 @@ __device__ __forceinline__ void read_state(const float4* src, StepState& S) {
   unpack_state(v, S);
 }
 
-// Asynchronous 16-byte global -> shared copies (L2 only, no L1 allocation).
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
-}
-
 // One lane's state: F4 float4 from a lane-interleaved global slot into its
 // lane-interleaved shared slot, as one commit group.
 template <int F4 = kStateF4>
@@ -984,25 +978,21 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
   using State = typename std::conditional<FORM == 1, UDState, StepState>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdSmem& B = *reinterpret_cast<BwdSmem*>(smem_raw);
-  load_tables(G, B.T);
-  for (int i = threadIdx.x; i < kAlignFloats; i += blockDim.x) B.align[i] = __ldg(a.align + i);
-  __syncthreads();
+  load_block_tables(G, B.T, B.align, a.align);
   const SmemTables& T = B.T;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   BwdWarpBufsT<F4>& W = reinterpret_cast<BwdWarpBufsT<F4>*>(smem_raw + sizeof(BwdSmem))[warp];
   // this warp's segment store: [step kk][float4 j][lane]
   float4* const gs = a.seg + ((int64_t)blockIdx.x * WARPS + warp) * (kCkptEvery * F4 * kWarp) + lane;
-  const int64_t n_chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
+  const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
   const int64_t N = a.n_tracks;
 #pragma unroll 1
-  for (;;) {
-    int64_t chunk = 0;
-    if (lane == 0) chunk = (int64_t)atomicAdd(a.work, 1u);
-    chunk = __shfl_sync(0xffffffffu, chunk, 0);
-    if (chunk >= n_chunks) break;
-    const int64_t slot = chunk * kWarp + lane;
-    if (slot >= N) continue;
+  for (bool first = true;; first = false) {
+    const int64_t item = next_item(a.work, n_items, first);
+    if (item < 0) break;
+    const int64_t slot = item * a.item_tracks + lane;
+    if (lane >= a.item_tracks || slot >= N) continue;
     const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
     const float g = __ldg(a.grad_chi2 + trk);
     const bool fitted = a.ndf[trk] > 0;
@@ -1164,10 +1154,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
 // memory.  tape_reverse_kernel then reverses the steps of each pass from the
 // last, copying each state from the tape into shared memory one step ahead;
 // it holds the reverse step's registers but does no forward work.
-// Tape layout: [pass][32-track work item][step][float4 j][lane], kTapeSteps
-// steps per work item, so that a warp's store or copy of float4 j of one step
-// moves 512 contiguous bytes.  Both kernels map processing slot k to work
-// item k / 32 and lane k % 32.  A track of more than kTapeSteps clusters (no
+// Tape layout: [pass][group of 32 slots][step][float4 j][slot in the group],
+// kTapeSteps steps per group, so that a full warp's store or copy of float4 j of
+// one step moves 512 contiguous bytes.  Processing slot k is in group k / 32 at
+// place k % 32, whatever the work items' size.  A track of more than kTapeSteps clusters (no
 // valid track has more than one per pad row) gets no gradient.
 constexpr int kTapeSteps = kMaxRows;
 
@@ -1175,9 +1165,10 @@ __host__ __device__ constexpr int64_t tape_float4s(int64_t n_tracks) {
   return 2 * ((n_tracks + kWarp - 1) / kWarp) * (int64_t)kTapeSteps * kStateF4 * kWarp;
 }
 
-// Float4 0 of step 0 of (pass, work item), offset by the lane.
-__device__ __forceinline__ int64_t tape_base(int pass, int64_t chunk, int64_t n_chunks, int lane) {
-  return (((int64_t)pass * n_chunks + chunk) * kTapeSteps) * (kStateF4 * kWarp) + lane;
+// Float4 0 of step 0 of (pass, processing slot).
+__device__ __forceinline__ int64_t tape_base(int pass, int64_t slot, int64_t n_tracks) {
+  const int64_t groups = (n_tracks + kWarp - 1) / kWarp;
+  return (((int64_t)pass * groups + slot / kWarp) * kTapeSteps) * (kStateF4 * kWarp) + slot % kWarp;
 }
 
 constexpr int kRecomputeWarps = 24;
@@ -1189,20 +1180,16 @@ __global__ void __launch_bounds__(kRecomputeWarps * 32, 1) recompute_kernel(cons
   constexpr int FIELD = (PHYS & 2) ? 1 : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdSmem& B = *reinterpret_cast<BwdSmem*>(smem_raw);
-  load_tables(G, B.T);
-  for (int i = threadIdx.x; i < kAlignFloats; i += blockDim.x) B.align[i] = __ldg(a.align + i);
-  __syncthreads();
+  load_block_tables(G, B.T, B.align, a.align);
   const SmemTables& T = B.T;
   const int lane = threadIdx.x & 31;
-  const int64_t n_chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
+  const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
 #pragma unroll 1
-  for (;;) {
-    int64_t chunk = 0;
-    if (lane == 0) chunk = (int64_t)atomicAdd(a.work, 1u);
-    chunk = __shfl_sync(0xffffffffu, chunk, 0);
-    if (chunk >= n_chunks) break;
-    const int64_t slot = chunk * kWarp + lane;
-    if (slot >= a.n_tracks) continue;
+  for (bool first = true;; first = false) {
+    const int64_t item = next_item(a.work, n_items, first);
+    if (item < 0) break;
+    const int64_t slot = item * a.item_tracks + lane;
+    if (lane >= a.item_tracks || slot >= a.n_tracks) continue;
     const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
     if (a.ndf[trk] <= 0) continue;
     const int begin = a.off[trk];
@@ -1215,7 +1202,7 @@ __global__ void __launch_bounds__(kRecomputeWarps * 32, 1) recompute_kernel(cons
       const int h0 = pass == 0 ? begin : begin + last;
       const int hd = pass == 0 ? 1 : -1;
       const float* ckp = a.ck + ((int64_t)pass * a.ck_slots + (begin >> kCkptShift) + trk) * kCkptFloats;
-      float4* const tp = a.tape + tape_base(pass, chunk, n_chunks, lane);
+      float4* const tp = a.tape + tape_base(pass, slot, a.n_tracks);
 #pragma unroll 1
       for (int s = 0; s < nseg; ++s) {
         const int i0 = s * kCkptEvery;
@@ -1254,24 +1241,20 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __gri
   constexpr int FIELD = (PHYS & 2) ? 1 : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdSmem& B = *reinterpret_cast<BwdSmem*>(smem_raw);
-  load_tables(G, B.T);
-  for (int i = threadIdx.x; i < kAlignFloats; i += blockDim.x) B.align[i] = __ldg(a.align + i);
-  __syncthreads();
+  load_block_tables(G, B.T, B.align, a.align);
   const SmemTables& T = B.T;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   float4 (*const st)[kStateF4][kWarp] =
       reinterpret_cast<float4 (*)[kStateF4][kWarp]>(smem_raw + sizeof(BwdSmem)) + 2 * warp;
-  const int64_t n_chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
+  const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
   const int64_t N = a.n_tracks;
 #pragma unroll 1
-  for (;;) {
-    int64_t chunk = 0;
-    if (lane == 0) chunk = (int64_t)atomicAdd(a.work, 1u);
-    chunk = __shfl_sync(0xffffffffu, chunk, 0);
-    if (chunk >= n_chunks) break;
-    const int64_t slot = chunk * kWarp + lane;
-    if (slot >= N) continue;
+  for (bool first = true;; first = false) {
+    const int64_t item = next_item(a.work, n_items, first);
+    if (item < 0) break;
+    const int64_t slot = item * a.item_tracks + lane;
+    if (lane >= a.item_tracks || slot >= N) continue;
     const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
     const float g = __ldg(a.grad_chi2 + trk);
     const bool fitted = a.ndf[trk] > 0;
@@ -1295,7 +1278,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __gri
         const int steps = last + 1;
         const int h0 = pass == 0 ? begin : begin + last;
         const int hd = pass == 0 ? 1 : -1;
-        const float4* const tp = a.tape + tape_base(pass, chunk, n_chunks, lane);
+        const float4* const tp = a.tape + tape_base(pass, slot, a.n_tracks);
         float pend0 = 0.0f, pend1 = 0.0f;  // gradient owed to the measurement of the step before
         const float2* const gmr = reinterpret_cast<const float2*>(a.grad_meas);
         const bool addg = pass == 0 && gmr != nullptr;
@@ -1352,86 +1335,51 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __gri
   }
 }
 
-template <int WARPS>
-constexpr size_t tape_reverse_smem_bytes() {
-  return sizeof(BwdSmem) + (size_t)WARPS * 2 * kStateF4 * kWarp * sizeof(float4);
-}
+constexpr size_t kTapeReverseWarpSmem = (size_t)2 * kStateF4 * kWarp * sizeof(float4);
 
-// Persistent launch of a kernel with `warps` warps per block and `smem` bytes
-// of shared memory (the grid cached per kernel).
-template <class K>
-cudaError_t launch_persistent(K kernel, int& cached, int warps, size_t smem, const BwdArgs& a, cudaStream_t s) {
-  if (cached == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, warps * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    cached = sms * per_sm;
-  }
-  const int64_t chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
-  const int64_t need = (chunks + warps - 1) / warps;
-  const int blocks = (int)(need < cached ? need : cached);
-  cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
+// Persistent launch of a kernel with up to `warps` warps per block, `block_smem`
+// bytes of shared memory per block and `warp_smem` per warp.
+template <class K, class A>
+cudaError_t launch_persistent(K kernel, Resident& r, int warps, size_t block_smem, size_t warp_smem, const A& a,
+                              cudaStream_t s) {
+  cudaError_t e = resident_blocks(kernel, warps * kWarp, block_smem + warps * warp_smem, r);
   if (e != cudaSuccess) return e;
-  kernel<<<blocks, warps * 32, smem, s>>>(a);
+  const WorkShape w = work_shape(a.n_tracks, r.blocks, warps, r.sms);
+  A b = a;
+  b.item_tracks = w.tracks;
+  if (needs_work_counter(w)) e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
+  if (e != cudaSuccess) return e;
+  kernel<<<w.blocks, w.warps * kWarp, block_smem + w.warps * warp_smem, s>>>(b);
   return cudaGetLastError();
 }
 
 template <int WARPS, int PHYS>
 cudaError_t launch_tape_backward_cfg(const BwdArgs& a, cudaStream_t s) {
-  static int g_rec = 0, g_rev = 0;
-  cudaError_t e = launch_persistent(recompute_kernel<PHYS>, g_rec, kRecomputeWarps, sizeof(BwdSmem), a, s);
+  static Resident g_rec, g_rev;
+  cudaError_t e = launch_persistent(recompute_kernel<PHYS>, g_rec, kRecomputeWarps, sizeof(BwdSmem), 0, a, s);
   if (e != cudaSuccess) return e;
-  return launch_persistent(tape_reverse_kernel<WARPS, PHYS>, g_rev, WARPS, tape_reverse_smem_bytes<WARPS>(), a, s);
+  return launch_persistent(tape_reverse_kernel<WARPS, PHYS>, g_rev, WARPS, sizeof(BwdSmem), kTapeReverseWarpSmem, a, s);
 }
 
-// Persistent grid of the backward (blocks resident at once over all SMs).
+// Blocks of the one-kernel backward resident at once.
 template <int WARPS, int PHYS, int FORM>
-cudaError_t backward_grid(int& grid) {
-  static int cached = 0;
-  if (cached == 0) {
-    constexpr int kThreads = WARPS * 32;
-    const size_t smem = backward_smem_bytes<WARPS, FORM>();
-    cudaError_t e = cudaFuncSetAttribute(backward_kernel<WARPS, PHYS, FORM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, backward_kernel<WARPS, PHYS, FORM>, kThreads, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    cached = sms * per_sm;
-  }
-  grid = cached;
-  return cudaSuccess;
+Resident& backward_resident() {
+  static Resident r;
+  return r;
 }
 
 template <int WARPS, int PHYS, int FORM>
 cudaError_t backward_store_cfg(int64_t& float4s) {
-  int grid = 0;
-  cudaError_t e = backward_grid<WARPS, PHYS, FORM>(grid);
-  float4s = (int64_t)grid * WARPS * kCkptEvery * (FORM ? kUDStateF4 : kStateF4) * kWarp;
+  Resident& r = backward_resident<WARPS, PHYS, FORM>();
+  cudaError_t e = resident_blocks(backward_kernel<WARPS, PHYS, FORM>, WARPS * kWarp, backward_smem_bytes<WARPS, FORM>(), r);
+  float4s = (int64_t)r.blocks * WARPS * kCkptEvery * (FORM ? kUDStateF4 : kStateF4) * kWarp;
   return e;
 }
 
 template <int WARPS, int PHYS, int FORM>
 cudaError_t launch_backward_cfg(const BwdArgs& a, cudaStream_t s) {
-  int grid = 0;
-  cudaError_t e = backward_grid<WARPS, PHYS, FORM>(grid);
-  if (e != cudaSuccess) return e;
-  const int64_t chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
-  const int64_t need = (chunks + WARPS - 1) / WARPS;
-  const int blocks = (int)(need < grid ? need : grid);
-  e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
-  if (e != cudaSuccess) return e;
-  backward_kernel<WARPS, PHYS, FORM><<<blocks, WARPS * 32, backward_smem_bytes<WARPS, FORM>(), s>>>(a);
-  return cudaGetLastError();
+  return launch_persistent(backward_kernel<WARPS, PHYS, FORM>, backward_resident<WARPS, PHYS, FORM>(), WARPS,
+                           sizeof(BwdSmem), sizeof(BwdWarpBufsT<FORM ? kUDStateF4 : kStateF4>), a, s);
 }
 
 // Warps per block of a backward launch: the configured shape in a uniform

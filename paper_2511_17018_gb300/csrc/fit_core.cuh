@@ -16,8 +16,8 @@
 // next cluster's sector frame if needed, analytic helix propagation to that pad
 // row with its Jacobian, L <- J L, two scalar Potter updates (y then z).
 //
-// Work mapping: a persistent grid; each warp takes 32-track work items from a
-// global counter and fits one track per lane.  While a lane computes the steps
+// Work mapping: a persistent grid; each warp takes work items of up to 32 tracks
+// (WorkShape, internal.h) and fits one track per lane.  While a lane computes the steps
 // of the current chunk, the warp's asynchronous copies (cp.async) bring the
 // next `RPS` clusters of all 32 tracks into the other half of a shared-memory
 // double buffer.  The alignment table and the geometry live in shared memory.
@@ -188,6 +188,61 @@ __device__ __forceinline__ void load_tables(const GeoRef& G, SmemTables& t) {
     t.rot_c[i] = G.rot_c[i];
     t.rot_s[i] = G.rot_s[i];
   }
+}
+
+// Asynchronous global -> shared copies (no register staging).
+__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem_src) : "memory");
+}
+// 16 bytes (L2 only, no L1 allocation).
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// The block's tables.  The alignment table (43.8 KB) is copied asynchronously in
+// 16-byte pieces while the geometry comes from the launch arguments: a block of
+// one warp otherwise waits for 342 loads in turn.  A table that is not 16-byte
+// aligned (the entry point without a handle takes 8-byte-aligned ones) is loaded
+// word by word.
+__device__ __forceinline__ void load_block_tables(const GeoRef& G, SmemTables& t, float* align, const float* src) {
+  if (src != nullptr) {
+    if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+      for (int i = threadIdx.x; i < kAlignFloats / 4; i += blockDim.x) cp_async16(align + 4 * i, src + 4 * i);
+    } else {
+      for (int i = threadIdx.x; i < kAlignFloats; i += blockDim.x) align[i] = __ldg(src + i);
+    }
+  }
+  cp_async_commit();
+  load_tables(G, t);
+  cp_async_wait<0>();
+  __syncthreads();
+}
+
+// The next work item of a warp (-1: none left): its place in the launch first,
+// then the work counter (see WorkShape in internal.h).  IN_ORDER: where the
+// launch does not place every item, all come from the counter; warps that start
+// together then fit items of one time frame, whose alignment table they share in
+// L1 (40 frames of 14,400 tracks on average: 1.24 ms, with the first items
+// spread over the SMs 1.26 ms; one frame of 400,000 tracks: 0.730 and 0.719 ms).
+template <bool IN_ORDER = false>
+__device__ __forceinline__ int64_t next_item(unsigned int* work, int64_t n_items, bool first) {
+  const int64_t placed = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const bool counted = placed < n_items;
+  int64_t item;
+  if (first && !(IN_ORDER && counted)) {
+    item = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  } else {
+    if (!counted) return -1;
+    unsigned k = 0;
+    if ((threadIdx.x & 31) == 0) k = atomicAdd(work, 1u);
+    item = (IN_ORDER ? 0 : placed) + (int64_t)__shfl_sync(0xffffffffu, k, 0);
+  }
+  return item < n_items ? item : -1;
 }
 
 // ---------------------------------------------------------------- one prediction step
@@ -590,15 +645,6 @@ struct TrackState {
   int used;
 };
 
-// Asynchronous 4-byte global -> shared copies (no register staging).
-__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
 // Double-buffered staging of RPS clusters for each of a warp's 32 tracks.  Row
 // pitch RPS + 1 keeps the consumer's reads (lane t reads row t) conflict-free.
 // rowsec travels as the aligned 32-bit word that contains it.
@@ -699,24 +745,21 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BlockSmem& B = *reinterpret_cast<BlockSmem*>(smem_raw);
   WarpStage<RPS>* stages = reinterpret_cast<WarpStage<RPS>*>(smem_raw + sizeof(BlockSmem));
-  load_tables(G, B.T);
-  for (int i = threadIdx.x; i < kAlignFloats; i += blockDim.x) B.align[i] = __ldg(a.align + i);
-  __syncthreads();
+  // (frames with tables of their own never read the block's)
+  load_block_tables(G, B.T, B.align, FRAMES && a.frame_align ? nullptr : a.align);
   const SmemTables& T = B.T;
   const int lane = threadIdx.x & 31;
   WarpStage<RPS>& st = stages[threadIdx.x >> 5];
   const unsigned rs_par0 = (unsigned)(((uintptr_t)a.rowsec >> 1) & 1u);
-  const int64_t n_chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
+  const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
 
 #pragma unroll 1
-  for (;;) {
-    // ---- take the next 32-track work item
-    int64_t chunk = 0;
-    if (lane == 0) chunk = (int64_t)atomicAdd(a.work, 1u);
-    chunk = __shfl_sync(0xffffffffu, chunk, 0);
-    if (chunk >= n_chunks) break;
-    const int64_t slot = chunk * kWarp + lane;
-    const bool have = slot < a.n_tracks;
+  for (bool first = true;; first = false) {
+    // ---- take the next work item
+    const int64_t item = next_item<FRAMES>(a.work, n_items, first);
+    if (item < 0) break;
+    const int64_t slot = item * a.item_tracks + lane;
+    const bool have = lane < a.item_tracks && slot < a.n_tracks;
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
 
     // ---- per-track input checks
@@ -932,24 +975,15 @@ cudaError_t launch_cfg(const FitArgs& a, cudaStream_t s) {
   constexpr int kThreads = WARPS * 32;
   const size_t smem = sizeof(BlockSmem) + WARPS * sizeof(WarpStage<RPS>);
   auto kernel = fit_kernel<RPS, WARPS, MINB, RECORD, FRAMES, PHYS, FORM>;
-  static int grid = 0;
-  if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    grid = sms * per_sm;
-  }
-  const int64_t chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
-  const int64_t need = (chunks + WARPS - 1) / WARPS;
-  const int blocks = (int)(need < grid ? need : grid);
-  cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
+  static Resident r;
+  cudaError_t e = resident_blocks(kernel, kThreads, smem, r);
   if (e != cudaSuccess) return e;
-  kernel<<<blocks, kThreads, smem, s>>>(a);
+  const WorkShape w = work_shape(a.n_tracks, r.blocks, WARPS, r.sms);
+  FitArgs b = a;
+  b.item_tracks = w.tracks;
+  if (needs_work_counter(w)) e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
+  if (e != cudaSuccess) return e;
+  kernel<<<w.blocks, w.warps * kWarp, sizeof(BlockSmem) + w.warps * sizeof(WarpStage<RPS>), s>>>(b);
   return cudaGetLastError();
 }
 

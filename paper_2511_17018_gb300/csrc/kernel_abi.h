@@ -89,6 +89,7 @@ struct FitArgs {
   int32_t mat;                 // material layers on (selects the kernel variant that crosses them)
   int32_t field;               // field map on (selects the kernel variant that follows it)
   int32_t form;                // factor of the covariance: 0 square root (L), 1 U-D (fast mode without material)
+  int32_t item_tracks;         // tracks per work item (1..32, set by the launcher)
 };
 
 // Arguments of one backward launch (same frame as the recorded fit).
@@ -116,6 +117,7 @@ struct BwdArgs {
   int32_t phys;                // physics of the recorded fit: bit 1 material layers, bit 2 the field map
   int32_t form;                // factor the fast one-kernel backward recomputes in: 0 square root (L), 1 U-D
   int32_t ck_form;             // factor the checkpoints hold: 0 L, 1 U-D (u, d)
+  int32_t item_tracks;         // tracks per work item (set by the launcher)
 };
 
 // Arguments of one smoother launch (same frame as the recorded fit).
@@ -142,6 +144,7 @@ struct SmoothArgs {
   float4* seg;                 // segment store, as for the adjoint
   int32_t ck_form;             // factor the checkpoints hold: 0 L, 1 U-D (u, d)
   int32_t mat;                 // material layers on (the recorded fit had them)
+  int32_t item_tracks;         // tracks per work item (set by the launcher)
 };
 
 // Error codes recorded in the device error word.

@@ -36,19 +36,65 @@ __global__ void __launch_bounds__(kThreads) length_hist(const int32_t* off, int3
     if (sh[b]) atomicAdd(&hist[b], sh[b]);
 }
 
+// start[b] = number of tracks longer than b (longest first), from the histogram
+// of 256 bins, by the first 256 threads of a block (all its threads call it).
+__device__ __forceinline__ void longest_first(const int* hist, int* start) {
+  __shared__ int warp_sum[kBins / 32];
+  const int t = threadIdx.x, lane = t & 31;
+  const int b = kBins - 1 - t;  // thread t owns bin 255 - t: an exclusive prefix sum from the longest bin
+  const int v = t < kBins ? hist[b] : 0;
+  int incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (t < kBins && lane == 31) warp_sum[t >> 5] = incl;
+  __syncthreads();
+  if (t < kBins) {
+    int before = incl - v;
+    for (int w = 0; w < (t >> 5); ++w) before += warp_sum[w];
+    start[b] = before;
+  }
+}
+
+// The whole ordering of a small batch in one block: histogram, prefix sum and
+// scatter, with nothing to clear beforehand.  Bound by its launch and two passes
+// of dependent loads.  For up to kSmallOrder tracks it replaces a memset and two
+// kernels (1,000 tracks: 14 us of kernels and two launch gaps).
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallItems = 16;
+constexpr int kSmallOrder = kSmallThreads * kSmallItems;
+
+__global__ void __launch_bounds__(kSmallThreads) length_order_small(const int32_t* off, int32_t n, int32_t* perm) {
+  __shared__ int hist[kBins];
+  __shared__ int cursor[kBins];
+  if (threadIdx.x < kBins) hist[threadIdx.x] = 0;
+  __syncthreads();
+  int bin[kSmallItems];
+#pragma unroll
+  for (int it = 0; it < kSmallItems; ++it) {
+    const int i = it * kSmallThreads + threadIdx.x;
+    bin[it] = i < n ? length_bin(off, i) : -1;
+  }
+#pragma unroll
+  for (int it = 0; it < kSmallItems; ++it)
+    if (bin[it] >= 0) atomicAdd(&hist[bin[it]], 1);
+  __syncthreads();
+  longest_first(hist, cursor);
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < kSmallItems; ++it)
+    if (bin[it] >= 0) perm[atomicAdd(&cursor[bin[it]], 1)] = it * kSmallThreads + threadIdx.x;
+}
+
 __global__ void __launch_bounds__(kThreads) length_scatter(const int32_t* off, int32_t n, const int32_t* hist,
                                                            int32_t* cursor, int32_t* perm) {
   __shared__ int start[kBins];
   __shared__ int local[kBins];
   __shared__ int base[kBins];
-  {
-    // start[b] = number of tracks longer than b (longest first)
-    const int b = threadIdx.x;
-    int acc = 0;
-    for (int L = kBins - 1; L > b; --L) acc += hist[L];
-    start[b] = acc;
-    local[b] = 0;
-  }
+  longest_first(hist, start);
+  local[threadIdx.x] = 0;
   __syncthreads();
   const int64_t first = (int64_t)blockIdx.x * kThreads * kItems;
   int bin[kItems], rank[kItems];
@@ -122,6 +168,10 @@ cudaError_t launch_frame_length_order(const int32_t* off, int32_t n_tracks, cons
 cudaError_t launch_length_order(const int32_t* off, int32_t n_tracks, int32_t* perm, int32_t* scratch,
                                 cudaStream_t s) {
   if (n_tracks <= 0) return cudaSuccess;
+  if (n_tracks <= kSmallOrder) {
+    length_order_small<<<1, kSmallThreads, 0, s>>>(off, n_tracks, perm);
+    return cudaGetLastError();
+  }
   cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int32_t) * 2 * kBins, s);
   if (e != cudaSuccess) return e;
   const int64_t blocks = ((int64_t)n_tracks + kThreads * kItems - 1) / (kThreads * kItems);

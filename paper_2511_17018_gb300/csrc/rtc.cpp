@@ -105,7 +105,7 @@ uint64_t fnv1a(const std::string& s, uint64_t h = 1469598103934665603ull) {
 struct Compiled {
   cudaLibrary_t lib = nullptr;
   cudaKernel_t kernel = nullptr;
-  std::unordered_map<int, int> grid;  // per device: resident blocks over all SMs
+  std::unordered_map<int, Resident> resident;  // per device
 };
 
 std::mutex g_mu;
@@ -249,8 +249,15 @@ Variant variant(const GeoConst& g, bool det, int rps, int warps, bool record, bo
            std::to_string(form) + ">";
   std::string opt;
   for (const std::string& x : options(det)) opt += x + " ";
+  // the device sources are part of the key: a cached CUBIN of other sources (an
+  // older library's) may take other launch arguments
+  static const uint64_t device_sources = [] {
+    uint64_t h = fnv1a("");
+    for (int i = 0; i < kRtcSourceCount; ++i) h = fnv1a(kRtcSources[i], h);
+    return h;
+  }();
   char keyb[32];
-  snprintf(keyb, sizeof keyb, "%016llx", (unsigned long long)fnv1a(v.expr, fnv1a(opt, fnv1a(v.src))));
+  snprintf(keyb, sizeof keyb, "%016llx", (unsigned long long)fnv1a(v.expr, fnv1a(opt, fnv1a(v.src, device_sources))));
   v.key = keyb;
   return v;
 }
@@ -331,30 +338,25 @@ tpcfit_status rtc_launch_fit(const GeoConst& g, bool det, int rps, int warps, co
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return TPCFIT_ECUDA;
-  int grid = 0;
+  Resident r;
   {
     std::lock_guard<std::mutex> lk(g_mu);
-    auto it = c->grid.find(dev);
-    if (it != c->grid.end()) grid = it->second;
+    auto it = c->resident.find(dev);
+    if (it != c->resident.end()) r = it->second;
   }
-  if (grid == 0) {
-    int sms = 0, per_sm = 0;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
-    if (e != cudaSuccess || per_sm < 1) return TPCFIT_ECUDA;
-    grid = sms * per_sm;
+  if (r.blocks == 0) {
+    if (resident_blocks(fn, threads, smem, r) != cudaSuccess) return TPCFIT_ECUDA;
     std::lock_guard<std::mutex> lk(g_mu);
-    c->grid[dev] = grid;
+    c->resident[dev] = r;
   }
-  const int64_t chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
-  const int64_t need = (chunks + warps - 1) / warps;
-  const int blocks = (int)(need < grid ? need : grid);
-  e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
-  if (e != cudaSuccess) return TPCFIT_ECUDA;
+  const WorkShape w = work_shape(a.n_tracks, r.blocks, warps, r.sms);
   FitArgs args = a;
+  args.item_tracks = w.tracks;
+  if (needs_work_counter(w)) e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
+  if (e != cudaSuccess) return TPCFIT_ECUDA;
   void* params[] = {&args};
-  e = cudaLaunchKernel(fn, dim3(blocks), dim3(threads), params, smem, s);
+  e = cudaLaunchKernel(fn, dim3(w.blocks), dim3(w.warps * kWarp), params,
+                       (size_t)kFitBlockSmemBytes + (size_t)w.warps * fit_warp_stage_bytes(rps), s);
   return e == cudaSuccess ? TPCFIT_OK : TPCFIT_ECUDA;
 }
 

@@ -241,23 +241,19 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
   const GeoRef& G = a.geo;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdSmem& B = *reinterpret_cast<BwdSmem*>(smem_raw);
-  load_tables(G, B.T);
-  for (int i = threadIdx.x; i < kAlignFloats; i += blockDim.x) B.align[i] = __ldg(a.align + i);
-  __syncthreads();
+  load_block_tables(G, B.T, B.align, a.align);
   const SmemTables& T = B.T;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   BwdWarpBufs& W = reinterpret_cast<BwdWarpBufs*>(smem_raw + sizeof(BwdSmem))[warp];
   float4* const gs = a.seg + ((int64_t)blockIdx.x * WARPS + warp) * (kCkptEvery * kStateF4 * kWarp) + lane;
-  const int64_t n_chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
+  const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
 #pragma unroll 1
-  for (;;) {
-    int64_t chunk = 0;
-    if (lane == 0) chunk = (int64_t)atomicAdd(a.work, 1u);
-    chunk = __shfl_sync(0xffffffffu, chunk, 0);
-    if (chunk >= n_chunks) break;
-    const int64_t slot = chunk * kWarp + lane;
-    if (slot >= a.n_tracks) continue;
+  for (bool first = true;; first = false) {
+    const int64_t item = next_item(a.work, n_items, first);
+    if (item < 0) break;
+    const int64_t slot = item * a.item_tracks + lane;
+    if (lane >= a.item_tracks || slot >= a.n_tracks) continue;
     const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
     const int begin = a.off[trk];
     const int end = a.off[trk + 1];
@@ -397,54 +393,38 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
 }
 
 #ifndef __CUDACC_RTC__
-template <int WARPS, bool MAT, bool STATES>
-cudaError_t smooth_grid(int& grid) {
-  static int cached = 0;
-  if (cached == 0) {
-    const size_t smem = smooth_smem_bytes<WARPS>();
-    cudaError_t e =
-        cudaFuncSetAttribute(smooth_kernel<WARPS, MAT, STATES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, smooth_kernel<WARPS, MAT, STATES>, WARPS * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    cached = sms * per_sm;
-  }
-  grid = cached;
-  return cudaSuccess;
-}
-
 constexpr int kSmoothWarps = 8;
 
-// Segment store (float4 count) the smoother needs (the larger of its variants).
+template <bool MAT, bool STATES>
+Resident& smooth_resident() {
+  static Resident r;
+  return r;
+}
+
+template <bool MAT, bool STATES>
+cudaError_t smooth_store_cfg(int& blocks) {
+  Resident& r = smooth_resident<MAT, STATES>();
+  const cudaError_t e = resident_blocks(smooth_kernel<kSmoothWarps, MAT, STATES>, kSmoothWarps * kWarp,
+                                        smooth_smem_bytes<kSmoothWarps>(), r);
+  if (r.blocks > blocks) blocks = r.blocks;
+  return e;
+}
+
+// Segment store (float4 count) the smoother needs (the largest of its variants).
 inline cudaError_t smooth_store(int64_t& float4s) {
-  int g[4] = {0, 0, 0, 0};
-  cudaError_t e = smooth_grid<kSmoothWarps, false, false>(g[0]);
-  if (e == cudaSuccess) e = smooth_grid<kSmoothWarps, true, false>(g[1]);
-  if (e == cudaSuccess) e = smooth_grid<kSmoothWarps, false, true>(g[2]);
-  if (e == cudaSuccess) e = smooth_grid<kSmoothWarps, true, true>(g[3]);
-  int gm = 0;
-  for (int i = 0; i < 4; ++i) gm = g[i] > gm ? g[i] : gm;
-  float4s = (int64_t)gm * kSmoothWarps * kCkptEvery * kStateF4 * kWarp;
+  int blocks = 0;
+  cudaError_t e = smooth_store_cfg<false, false>(blocks);
+  if (e == cudaSuccess) e = smooth_store_cfg<true, false>(blocks);
+  if (e == cudaSuccess) e = smooth_store_cfg<false, true>(blocks);
+  if (e == cudaSuccess) e = smooth_store_cfg<true, true>(blocks);
+  float4s = (int64_t)blocks * kSmoothWarps * kCkptEvery * kStateF4 * kWarp;
   return e;
 }
 
 template <bool MAT, bool STATES>
 cudaError_t launch_smooth_cfg(const SmoothArgs& a, cudaStream_t s) {
-  int grid = 0;
-  cudaError_t e = smooth_grid<kSmoothWarps, MAT, STATES>(grid);
-  if (e != cudaSuccess) return e;
-  const int64_t chunks = ((int64_t)a.n_tracks + kWarp - 1) / kWarp;
-  const int64_t need = (chunks + kSmoothWarps - 1) / kSmoothWarps;
-  const int blocks = (int)(need < grid ? need : grid);
-  e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
-  if (e != cudaSuccess) return e;
-  smooth_kernel<kSmoothWarps, MAT, STATES><<<blocks, kSmoothWarps * 32, smooth_smem_bytes<kSmoothWarps>(), s>>>(a);
-  return cudaGetLastError();
+  return launch_persistent(smooth_kernel<kSmoothWarps, MAT, STATES>, smooth_resident<MAT, STATES>(), kSmoothWarps,
+                           sizeof(BwdSmem), sizeof(BwdWarpBufs), a, s);
 }
 
 inline cudaError_t launch_smooth(const SmoothArgs& a, cudaStream_t s) {
