@@ -214,18 +214,24 @@ long long tpcfit_rtc_compile_count(void);
 /* Log of the last NVRTC compilation (empty if none); valid until the next one. */
 const char* tpcfit_rtc_log(void);
 
-/* Record checkpoints for the adjoint (record = 1) or not (0, default).  With
- * recording on, tpcfit_fit also stores the filter state before every 16th step
- * of both passes (about 8 floats per cluster, handle-owned, grown as needed) so
- * that tpcfit_fit_backward can follow.  Any tpcfit_fit call replaces the
- * recording. */
+/* Record the fit for the adjoint and the smoother (record = 1) or not (0,
+ * default).  With recording on, tpcfit_fit also writes a tape of filter states,
+ * handle-owned and grown as needed, so that tpcfit_fit_backward can follow: the
+ * state before every step of both passes (U-D form: 176 bytes per cluster, or
+ * 96 with every second state, from 38,913 tracks on 152 SMs; deterministic mode
+ * and material layers: 256 bytes).  Where the tape would take more than half of
+ * the free device memory, and in the forms without one (several lanes per track;
+ * the fast square-root form without material), the fit leaves checkpoints
+ * instead: the state before every 16th step (about 8 floats per cluster, also
+ * handle-owned).  Any tpcfit_fit call replaces the recording. */
 tpcfit_status tpcfit_set_record(tpcfit_handle* h, int record);
 
-/* Launch configuration of the adjoint's reverse: warps per block (4, 8, 10 or
- * 12; default 8).  Each resident warp owns 8-12 KB of shared memory that holds
- * the states it copies ahead (and, in fast mode without material, a segment
- * store in device memory that the handle allocates on the first backward).
- * Results do not depend on it.  EINVAL for other values. */
+/* Launch configuration of the adjoint's reverse from checkpoints: warps per
+ * block (4, 8, 10 or 12; default 8).  Each resident warp owns 8-12 KB of shared
+ * memory that holds the states it copies ahead, and a segment store in device
+ * memory that the handle allocates on the first backward.  The reverse from the
+ * tape (tpcfit_set_record) has its own shapes.  Results do not depend on it.
+ * EINVAL for other values. */
 tpcfit_status tpcfit_set_backward_config(tpcfit_handle* h, int warps_per_block);
 
 /* Factor of the covariance that the fast fit without material layers carries:
@@ -283,17 +289,14 @@ tpcfit_status tpcfit_set_det_reduction(tpcfit_handle* h, int method);
  *   grad_align: float [36][152][2], dL/d(dy, dz) of the alignment offsets;
  *   grad_seeds: float [5][n_tracks], dL/dseed;
  *   grad_meas:  float [n_hits][2], dL/d(measured y, z) per cluster, or NULL.
- * The backward recomputes each 16-step segment from its checkpoint and runs
- * the hand-written reverse of every step, copying the state before each step
- * into shared memory one step ahead.  Fast mode without material layers
- * recomputes into a per-warp segment store in the same kernel, in the factor
- * form tpcfit_set_backward_form chose; the
- * deterministic mode and the material layers replay the segments in a kernel
- * of their own onto a tape of every step's state (about 40 MB per 1,000
- * tracks, handle-owned, grown as needed) and reverse from it.  It follows the
+ * The backward runs the hand-written reverse of every step, copying the state
+ * before each step into shared memory ahead of its use: from the recorded fit's
+ * tape (with every second state on it, the others are recomputed one step at a
+ * time), or, from checkpoints, recomputing each 16-step segment into a per-warp
+ * segment store first, in the factor form tpcfit_set_backward_form chose (the
+ * deterministic mode and the material layers: square root).  It follows the
  * field map and the material layers (tpcfit_set_field_map,
- * tpcfit_set_material).  Tracks of more than 152 clusters get no gradient in
- * the taped cases.  Fast mode accumulates grad_align with
+ * tpcfit_set_material).  Fast mode accumulates grad_align with
  * atomics; deterministic mode writes per-cluster gradients and reduces them
  * per (sector, row) so that grad_align is bitwise reproducible, by the method
  * tpcfit_set_det_reduction chose.  Tracks with ndf <= 0 contribute 0. */

@@ -361,27 +361,6 @@ struct StepState {
   int sec;
 };
 
-__device__ __forceinline__ void load_ckpt(const float* src, StepState& S) {
-  const float4* s4 = reinterpret_cast<const float4*>(src);
-  float v[32];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const float4 f = __ldg(s4 + j);
-    v[4 * j] = f.x;
-    v[4 * j + 1] = f.y;
-    v[4 * j + 2] = f.z;
-    v[4 * j + 3] = f.w;
-  }
-#pragma unroll
-  for (int c = 0; c < 5; ++c) S.p[c] = v[c];
-#pragma unroll
-  for (int i = 0; i < 5; ++i)
-#pragma unroll
-    for (int c = 0; c < 5; ++c) S.L[i][c] = v[5 + 5 * i + c];
-  S.x = v[30];
-  S.sec = __float_as_int(v[31]);
-}
-
 // A checkpoint of the U-D fit, loaded as if it held L (u in rows 0-1, d in
 // row 2): turned into the square-root factor L = U sqrt(D), upper triangular.
 __device__ __forceinline__ void sqrt_from_ud_ckpt(StepState& S) {
@@ -938,7 +917,7 @@ __device__ __forceinline__ void accumulate_meas_grad(const BwdArgs& a, int pass,
   }
 }
 
-// Shared memory of a backward block: geometry tables, the alignment table
+// Shared memory of a backward block (from checkpoints): geometry tables, the alignment table
 // and, per warp, a double buffer for the state before the step being reversed
 // and a buffer for the next segment's checkpoint (all [float4 j][lane]).
 struct BwdSmem {
@@ -965,17 +944,18 @@ constexpr size_t backward_smem_bytes() {
 // first, each state copied into shared memory asynchronously one step ahead.
 // Clusters are loaded one step ahead as well; the next segment's checkpoint
 // is copied while the current segment is reversed.
-// PHYS: bit 1 the material layers, bit 2 the field map.  FORM: the factor the
-// segments are recomputed in, 0 the fit's square-root factor L, 1 U-D (no
-// material layers; the checkpoint's L is converted where a segment starts).
+// Fast mode without material layers.  PHYS: bit 2 the field map.  FORM: the factor
+// the segments are recomputed in, 0 the fit's square-root factor L, 1 U-D (a
+// checkpoint's L is converted where a segment starts).
 template <int WARPS, int PHYS, int FORM = 0>
 __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_constant__ BwdArgs a) {
   const GeoRef& G = a.geo;
-  constexpr bool MAT = (PHYS & 1) != 0;
   constexpr int FIELD = (PHYS & 2) ? 1 : 0;
-  static_assert(FORM == 0 || !MAT, "the U-D backward runs without material layers");
   constexpr int F4 = FORM ? kUDStateF4 : kStateF4;
   using State = typename std::conditional<FORM == 1, UDState, StepState>::type;
+  // after a taped fit only the items that found no room on the tape are left
+  // (none, unless tracks overlap or have more than 255 clusters)
+  if (a.tape_item && a.work[kWorkMissing] == 0) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdSmem& B = *reinterpret_cast<BwdSmem*>(smem_raw);
   load_block_tables(G, B.T, B.align, a.align);
@@ -991,6 +971,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
   for (bool first = true;; first = false) {
     const int64_t item = next_item(a.work, n_items, first);
     if (item < 0) break;
+    if (a.tape_item && a.tape_item[item].x >= 0) continue;
     const int64_t slot = item * a.item_tracks + lane;
     if (lane >= a.item_tracks || slot >= N) continue;
     const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
@@ -1062,9 +1043,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
             decode_hit(B.align, cur, m0, m1, row, sec);
             store_state(gs + kk * (F4 * kWarp), S);
             if constexpr (FORM == 1)
-              step_fwd_ud<FIELD>(G, T, S, my, mz, i == 0, pass == 0, row, side_sector(sec), m0, m1);
+              step_fwd_ud<FIELD>(G, T, S, my, mz, i == 0, pass == 0, T.row_x[row], side_sector(sec), m0, m1);
             else
-              step_fwd<MAT, FIELD>(G, T, S, my, mz, i == 0, pass == 0, row, side_sector(sec), m0, m1);
+              step_fwd<false, FIELD>(G, T, S, my, mz, i == 0, pass == 0, row, side_sector(sec), m0, m1);
           }
           // the states just stored are read back by this thread's copies below
           __threadfence_block();
@@ -1112,18 +1093,14 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
             float b_mc[2], b_mp[2];
             if constexpr (FORM == 1) {
               step_rev_ud<FIELD>(G, T, &W.st[kk & 1][0][lane], mpy, mpz, T.row_x[prow], side_sector(psec), i == 0,
-                                 pass == 0, row, side_sector(sec), m0, m1, b_p, b_u, b_d, b_chi,
+                                 pass == 0, T.row_x[row], side_sector(sec), m0, m1, b_p, b_u, b_d, b_chi,
                                  [&](float g0, float g1) {
                                    accumulate_meas_grad(a, pass, h, row, sec, g0 + pend0, g1 + pend1, gcur);
                                  },
                                  b_mp);
             } else {
-              if (MAT)
-                step_rev_mat<FIELD>(G, T, &W.st[kk & 1][0][lane], mpy, mpz, i == 0, pass == 0, row, side_sector(sec), m0,
-                                    m1, b_p, b_L, b_chi, b_mc, b_mp);
-              else
-                step_rev<FIELD>(G, T, &W.st[kk & 1][0][lane], mpy, mpz, i == 0, pass == 0, row, side_sector(sec), m0, m1,
-                                b_p, b_L, b_chi, b_mc, b_mp);
+              step_rev<FIELD>(G, T, &W.st[kk & 1][0][lane], mpy, mpz, i == 0, pass == 0, row, side_sector(sec), m0, m1,
+                              b_p, b_L, b_chi, b_mc, b_mp);
               accumulate_meas_grad(a, pass, h, row, sec, b_mc[0] + pend0, b_mc[1] + pend1, gcur);
             }
             pend0 = b_mp[0];
@@ -1148,92 +1125,216 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
 }
 
 // ---------------------------------------------------------------- the tape
-// The backward in two kernels.  recompute_kernel replays every 16-step
-// segment of both passes from its checkpoint (the fit's own arithmetic, at the
-// fit's occupancy) and writes the state before each step to a tape in device
-// memory.  tape_reverse_kernel then reverses the steps of each pass from the
-// last, copying each state from the tape into shared memory one step ahead;
-// it holds the reverse step's registers but does no forward work.
-// Tape layout: [pass][group of 32 slots][step][float4 j][slot in the group],
-// kTapeSteps steps per group, so that a full warp's store or copy of float4 j of
-// one step moves 512 contiguous bytes.  Processing slot k is in group k / 32 at
-// place k % 32, whatever the work items' size.  A track of more than kTapeSteps clusters (no
-// valid track has more than one per pad row) gets no gradient.
-constexpr int kTapeSteps = kMaxRows;
+// Reverse of both passes from the recorded fit's tape (inward pass first).  The
+// states are copied into shared memory ahead of their use, as contiguous rows.
+// The steps of a pass run over the warp's longest track for all its lanes
+// together (a lane of a shorter track joins when its last step comes), so that
+// lanes of different lengths stay converged.
 
-__host__ __device__ constexpr int64_t tape_float4s(int64_t n_tracks) {
-  return 2 * ((n_tracks + kWarp - 1) / kWarp) * (int64_t)kTapeSteps * kStateF4 * kWarp;
+// The lane's float4 of row 0 of an item.
+__device__ __forceinline__ const float4* tape_row0(const float4* tape, int2 place, int pitch, int lane) {
+  return tape + (int64_t)place.x * pitch + lane;
 }
 
-// Float4 0 of step 0 of (pass, processing slot).
-__device__ __forceinline__ int64_t tape_base(int pass, int64_t slot, int64_t n_tracks) {
-  const int64_t groups = (n_tracks + kWarp - 1) / kWarp;
-  return (((int64_t)pass * groups + slot / kWarp) * kTapeSteps) * (kStateF4 * kWarp) + slot % kWarp;
+template <int ROWS>
+__device__ __forceinline__ void copy_rows(float4* sdst, const float4* src, int pitch) {
+#pragma unroll
+  for (int j = 0; j < ROWS; ++j) cp_async16(sdst + j * kWarp, src + j * pitch);
 }
 
-constexpr int kRecomputeWarps = 24;
+// U-D form (fast mode without material layers).  The fit stores the state before
+// every EVERY-th step; with EVERY = 2 the odd states are recomputed from the even
+// ones.  Per warp, EVERY steps ("a group") at a time: three groups in shared
+// memory, the one being reversed, the one before it (its last cluster is the
+// previous cluster of this one's first step) and one on its way.
+//
+// EVERY = 1 writes and reads 176 bytes a cluster and recomputes nothing: for
+// batches that wait for their longest tracks rather than for memory.  EVERY = 2
+// halves the states: the fit of 400,000 tracks writes at 4 TB/s, which with every
+// state takes 1.54 ms (0.73 unrecorded).  Clusters are stored once for both
+// passes, with the alignment taken off, so the reverse needs neither the hits nor
+// the alignment table.
+template <int EVERY>
+struct TapeGroup {
+  float4 state[kUDRows][kWarp];
+  float4 cluster[EVERY][kWarp];
+};
+template <int EVERY>
+struct TapeWarpUD {
+  TapeGroup<EVERY> g[3];
+  float4 odd[EVERY - 1 ? kUDRows : 1][kWarp];  // the recomputed state
+};
+template <>
+struct TapeWarpUD<1> {
+  TapeGroup<1> g[3];
+};
 
-template <int PHYS>
-__global__ void __launch_bounds__(kRecomputeWarps * 32, 1) recompute_kernel(const __grid_constant__ BwdArgs a) {
+template <int WARPS, int PHYS, int EVERY>
+__global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_ud_kernel(const __grid_constant__ BwdArgs a) {
   const GeoRef& G = a.geo;
-  constexpr bool MAT = (PHYS & 1) != 0;
   constexpr int FIELD = (PHYS & 2) ? 1 : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  BwdSmem& B = *reinterpret_cast<BwdSmem*>(smem_raw);
-  load_block_tables(G, B.T, B.align, a.align);
-  const SmemTables& T = B.T;
+  SmemTables& T = *reinterpret_cast<SmemTables*>(smem_raw);
+  load_tables(G, T);
+  __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
+  TapeWarpUD<EVERY>& W = reinterpret_cast<TapeWarpUD<EVERY>*>(smem_raw + sizeof(SmemTables))[threadIdx.x >> 5];
+  const int pitch = a.item_tracks;
+  const int64_t n_items = ((int64_t)a.n_tracks + pitch - 1) / pitch;
+  const int64_t N = a.n_tracks;
 #pragma unroll 1
   for (bool first = true;; first = false) {
     const int64_t item = next_item(a.work, n_items, first);
     if (item < 0) break;
-    const int64_t slot = item * a.item_tracks + lane;
-    if (lane >= a.item_tracks || slot >= a.n_tracks) continue;
-    const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
-    if (a.ndf[trk] <= 0) continue;
-    const int begin = a.off[trk];
-    const int last = a.ck_last[trk];
-    const int steps = last + 1;
-    if (steps > kTapeSteps) continue;
-    const int nseg = (steps + kCkptEvery - 1) / kCkptEvery;
+    const int2 place = a.tape_item[item];
+    if (place.x < 0) continue;  // left to backward_kernel
+    const int64_t slot = item * pitch + lane;
+    const bool have = lane < pitch && slot < N;
+    const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
+    const bool fitted = have && a.ndf[trk] > 0;
+    const float g = fitted ? __ldg(a.grad_chi2 + trk) : 0.0f;
+    const int begin = have ? a.off[trk] : 0;
+    const int steps = fitted ? a.ck_last[trk] + 1 : 0;
+    const int most = __reduce_max_sync(0xffffffffu, steps);
+    const float4* const row0 = tape_row0(a.tape, place, pitch, lane);
+    float b_p[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      const int h0 = pass == 0 ? begin : begin + last;
-      const int hd = pass == 0 ? 1 : -1;
-      const float* ckp = a.ck + ((int64_t)pass * a.ck_slots + (begin >> kCkptShift) + trk) * kCkptFloats;
-      float4* const tp = a.tape + tape_base(pass, slot, a.n_tracks);
-#pragma unroll 1
-      for (int s = 0; s < nseg; ++s) {
-        const int i0 = s * kCkptEvery;
-        const int cnt = min(kCkptEvery, steps - i0);
-        StepState S;
-        load_ckpt(ckp + (int64_t)s * kCkptFloats, S);
-        if (a.ck_form == 1) sqrt_from_ud_ckpt(S);
-        float my = 0.0f, mz = 0.0f;
-        if (i0 > 0) {
-          int row, sec;
-          decode_hit(B.align, load_hit(a, h0 + hd * (i0 - 1)), my, mz, row, sec);
+    for (int pass = 1; pass >= 0; --pass) {
+      float b_u[10], b_d[5];
+#pragma unroll
+      for (int e = 0; e < 10; ++e) b_u[e] = 0.0f;
+#pragma unroll
+      for (int c = 0; c < 5; ++c) b_d[c] = 0.0f;
+      const float b_chi = pass == 1 ? g : 0.0f;
+      // the outward pass adds to the inward pass's gradient of each cluster:
+      // that value is read one reversed step ahead
+      const bool addg = pass == 0 && a.grad_meas != nullptr;
+      const float2* const gmr = reinterpret_cast<const float2*>(a.grad_meas);
+      const int h0 = pass == 0 ? begin : begin + steps - 1, hd = pass == 0 ? 1 : -1;
+      float2 gnx = addg && steps > 0 ? gmr[h0 + hd * (steps - 1)] : make_float2(0.0f, 0.0f);
+      float pend0 = 0.0f, pend1 = 0.0f;  // gradient owed to the measurement of the step before
+      // step i of the pass: cluster row c0 + cd i, state i / EVERY
+      const float4* const clusters = row0 + (pass == 0 ? 0 : steps - 1) * pitch;
+      const int cd = hd * pitch;
+      const float4* const states = row0 + (place.y + kUDRows * pass * (int)tape_states(place.y, EVERY)) * pitch;
+      auto fetch = [&](TapeGroup<EVERY>& to, int grp) {
+        const int i = grp * EVERY;
+        if (i >= 0 && i < steps) {
+          copy_rows<kUDRows>(&to.state[0][lane], states + grp * (kUDRows * pitch), pitch);
+#pragma unroll
+          for (int k = 0; k < EVERY; ++k)
+            if (k == 0 || i + k < steps) cp_async16(&to.cluster[k][lane], clusters + (i + k) * cd);
         }
-        HitRaw nx = load_hit(a, h0 + hd * i0);
+        cp_async_commit();
+      };
+      const int last_grp = most > 0 ? (most - 1) / EVERY : -1;
+      fetch(W.g[0], last_grp);
+      fetch(W.g[1], last_grp - 1);
+      int s0 = 0, s1 = 1, s2 = 2;  // places of groups grp, grp - 1, grp - 2
 #pragma unroll 1
-        for (int kk = 0; kk < cnt; ++kk) {
-          const int i = i0 + kk;
-          const HitRaw cur = nx;
-          if (kk + 1 < cnt) nx = load_hit(a, h0 + hd * (i + 1));
-          float m0, m1;
-          int row, sec;
-          decode_hit(B.align, cur, m0, m1, row, sec);
-          store_state(tp + (int64_t)i * (kStateF4 * kWarp), S);
-          step_fwd<MAT, FIELD>(G, T, S, my, mz, i == 0, pass == 0, row, side_sector(sec), m0, m1);
+      for (int i = most - 1; i >= 0; --i) {
+        const int k = EVERY == 1 ? 0 : i & 1;  // place in the group
+        if (EVERY == 1 || k == 1 || i == most - 1) {
+          fetch(W.g[s2], i / EVERY - 2);
+          cp_async_wait<1>();  // groups i / EVERY and the one before are in place
+        }
+        if (i < steps) {
+          const float4* src = &W.g[s0].state[0][lane];
+          const float4 cur = W.g[s0].cluster[k][lane];
+          float4 prv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          if (k > 0)
+            prv = W.g[s0].cluster[0][lane];
+          else if (i > 0)
+            prv = W.g[s1].cluster[EVERY - 1][lane];
+          const int rs = __float_as_int(cur.w);
+          if constexpr (EVERY == 2) {
+            if (k == 1) {  // the state before this step: forward of the step before it (cluster prv)
+              UDState S;
+              read_state_ud<false>(src, S);
+              float4 pp = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+              if (i > 1) pp = W.g[s1].cluster[EVERY - 1][lane];
+              S.x = pp.z;
+              S.sec = side_sector(__float_as_int(pp.w) & 63);
+              step_fwd_ud<FIELD>(G, T, S, pp.x, pp.y, i == 1, pass == 0, prv.z,
+                                 side_sector(__float_as_int(prv.w) & 63), prv.x, prv.y);
+              src = &W.odd[0][lane];
+              store_state(&W.odd[0][lane], S);
+            }
+          }
+          const float2 gcur = gnx;
+          const int h = h0 + hd * i;
+          if (addg && i > 0) gnx = gmr[h - hd];
+          float b_mp[2];
+          step_rev_ud<FIELD>(G, T, src, prv.x, prv.y, prv.z, side_sector(__float_as_int(prv.w) & 63), i == 0,
+                             pass == 0, cur.z, side_sector(rs & 63), cur.x, cur.y, b_p, b_u, b_d, b_chi,
+                             [&](float g0, float g1) {
+                               accumulate_meas_grad(a, pass, h, rs >> 6, rs & 63, g0 + pend0, g1 + pend1, gcur);
+                             },
+                             b_mp);
+          pend0 = b_mp[0];
+          pend1 = b_mp[1];
+        }
+        if (k == 0) {
+          const int t = s0;
+          s0 = s1;
+          s1 = s2;
+          s2 = t;
         }
       }
+      // the inward pass starts from the outward result with the factor reset:
+      // b_p carries over, b_u and b_d do not
+      cp_async_wait<0>();
     }
+    if (!have) continue;
+    if (!fitted && a.grad_meas) {
+      const int end = a.off[trk + 1];
+      for (int h = begin; h < end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
+    }
+#pragma unroll
+    for (int c = 0; c < 5; ++c) a.grad_seeds[(int64_t)c * N + trk] = b_p[c];
   }
 }
 
-// The reverse of both passes from the tape (inward pass first); the same
-// reverse steps, cluster loads and gradient accumulation as backward_kernel.
+constexpr size_t kTapeWarpSmemSqrt = sizeof(float4) * 2 * kSqrtRows * kWarp;
+
+// The states of steps [i0, i0 + cnt) of a pass, recomputed from the checkpoint of
+// step i0 into the warp's segment store (gs: this lane's float4 0 of it).  h: the
+// cluster of step 0, hd: from one step's cluster to the next.  Not inlined: it
+// runs for the items without a place on the tape only.
+template <bool MAT, int FIELD>
+__device__ __noinline__ void recompute_segment(const BwdArgs& a, const SmemTables& T, const float* align,
+                                               const float* ck, float4* gs, int h, int hd, int i0, int cnt, bool conv) {
+  StepState S;
+  {
+    const float4* c4 = reinterpret_cast<const float4*>(ck);
+    float v[32];
+#pragma unroll
+    for (int j = 0; j < kStateF4; ++j) {
+      const float4 f = __ldg(c4 + j);
+      v[4 * j] = f.x;
+      v[4 * j + 1] = f.y;
+      v[4 * j + 2] = f.z;
+      v[4 * j + 3] = f.w;
+    }
+    unpack_state(v, S);
+  }
+  float my = 0.0f, mz = 0.0f;
+  if (i0 > 0) {
+    int row, sec;
+    decode_hit(align, load_hit(a, h + hd * (i0 - 1)), my, mz, row, sec);
+  }
+#pragma unroll 1
+  for (int kk = 0; kk < cnt; ++kk) {
+    float m0, m1;
+    int row, sec;
+    decode_hit(align, load_hit(a, h + hd * (i0 + kk)), m0, m1, row, sec);
+    store_state(gs + kk * (kStateF4 * kWarp), S);
+    step_fwd<MAT, FIELD>(a.geo, T, S, my, mz, i0 + kk == 0, conv, row, side_sector(sec), m0, m1);
+  }
+}
+
+// Square-root form (deterministic mode; material layers).  An item without a place
+// on the tape is recomputed segment by segment instead, in the same reverse loop.
 template <int WARPS, int PHYS>
 __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __grid_constant__ BwdArgs a) {
   const GeoRef& G = a.geo;
@@ -1244,98 +1345,116 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __gri
   load_block_tables(G, B.T, B.align, a.align);
   const SmemTables& T = B.T;
   const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  float4 (*const st)[kStateF4][kWarp] =
-      reinterpret_cast<float4 (*)[kStateF4][kWarp]>(smem_raw + sizeof(BwdSmem)) + 2 * warp;
-  const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
+  float4 (*const st)[kSqrtRows][kWarp] =
+      reinterpret_cast<float4 (*)[kSqrtRows][kWarp]>(smem_raw + sizeof(BwdSmem)) + 2 * (threadIdx.x >> 5);
+  float4* const gs =
+      a.seg + ((int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5)) * (kCkptEvery * kStateF4 * kWarp) + lane;
+  const int pitch = a.item_tracks;
+  const int64_t n_items = ((int64_t)a.n_tracks + pitch - 1) / pitch;
   const int64_t N = a.n_tracks;
 #pragma unroll 1
   for (bool first = true;; first = false) {
     const int64_t item = next_item(a.work, n_items, first);
     if (item < 0) break;
-    const int64_t slot = item * a.item_tracks + lane;
-    if (lane >= a.item_tracks || slot >= N) continue;
-    const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
-    const float g = __ldg(a.grad_chi2 + trk);
-    const bool fitted = a.ndf[trk] > 0;
+    const int2 place = a.tape_item ? a.tape_item[item] : make_int2(-1, 0);
+    const bool taped = place.x >= 0;
+    const int64_t slot = item * pitch + lane;
+    const bool have = lane < pitch && slot < N;
+    const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
+    const bool fitted = have && a.ndf[trk] > 0;
+    const float g = fitted ? __ldg(a.grad_chi2 + trk) : 0.0f;
+    const int begin = have ? a.off[trk] : 0;
+    const int steps = fitted ? a.ck_last[trk] + 1 : 0;
+    const int most = __reduce_max_sync(0xffffffffu, steps);
     float b_p[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    const int begin = fitted ? a.off[trk] : 0;
-    const int last = fitted ? a.ck_last[trk] : 0;
-    if (fitted && last + 1 <= kTapeSteps) {
-      float b_L[5][5];         // FORM 0: adjoint of the square-root factor
-      float b_u[10], b_d[5];   // FORM 1: adjoint of the U-D factor
 #pragma unroll 1
-      for (int pass = 1; pass >= 0; --pass) {
+    for (int pass = 1; pass >= 0; --pass) {
+      float b_L[5][5];
 #pragma unroll
-        for (int i = 0; i < 5; ++i)
+      for (int i = 0; i < 5; ++i)
 #pragma unroll
-          for (int c = 0; c < 5; ++c) b_L[i][c] = 0.0f;
-#pragma unroll
-        for (int e = 0; e < 10; ++e) b_u[e] = 0.0f;
-#pragma unroll
-        for (int c = 0; c < 5; ++c) b_d[c] = 0.0f;
-        const float b_chi = pass == 1 ? g : 0.0f;
-        const int steps = last + 1;
-        const int h0 = pass == 0 ? begin : begin + last;
-        const int hd = pass == 0 ? 1 : -1;
-        const float4* const tp = a.tape + tape_base(pass, slot, a.n_tracks);
-        float pend0 = 0.0f, pend1 = 0.0f;  // gradient owed to the measurement of the step before
-        const float2* const gmr = reinterpret_cast<const float2*>(a.grad_meas);
-        const bool addg = pass == 0 && gmr != nullptr;
-        float2 gnx = addg ? gmr[h0 + hd * (steps - 1)] : make_float2(0.0f, 0.0f);
-        fetch_state(&st[(steps - 1) & 1][0][lane], tp + (int64_t)(steps - 1) * (kStateF4 * kWarp));
-        float m0, m1;
-        int row, sec;
-        decode_hit(B.align, load_hit(a, h0 + hd * (steps - 1)), m0, m1, row, sec);
-        HitRaw pv{};
-        if (steps > 1) pv = load_hit(a, h0 + hd * (steps - 2));
+        for (int c = 0; c < 5; ++c) b_L[i][c] = 0.0f;
+      const float b_chi = pass == 1 ? g : 0.0f;
+      const int h0 = pass == 0 ? begin : begin + steps - 1, hd = pass == 0 ? 1 : -1;
+      const bool addg = pass == 0 && a.grad_meas != nullptr;
+      const float2* const gmr = reinterpret_cast<const float2*>(a.grad_meas);
+      float2 gnx = addg && steps > 0 ? gmr[h0 + hd * (steps - 1)] : make_float2(0.0f, 0.0f);
+      float pend0 = 0.0f, pend1 = 0.0f;  // gradient owed to the measurement of the step before
+      float m0 = 0.0f, m1 = 0.0f;
+      int row = 0, sec = 0;
+      if (steps > 0) decode_hit(B.align, load_hit(a, h0 + hd * (steps - 1)), m0, m1, row, sec);
+      HitRaw pv{};
+      if (steps > 1) pv = load_hit(a, h0 + hd * (steps - 2));
+      // steps [lo, hi) at a time: the whole pass from the tape, else a segment
+      int hi = most;
 #pragma unroll 1
-        for (int i = steps - 1; i >= 0; --i) {
-          const int h = h0 + hd * i;
-          if (i > 0) {
-            fetch_state(&st[(i - 1) & 1][0][lane], tp + (int64_t)(i - 1) * (kStateF4 * kWarp));
-            cp_async_wait<1>();
-          } else {
-            cp_async_wait<0>();
-          }
-          float mpy = 0.0f, mpz = 0.0f;
-          int prow = 0, psec = 0;
-          if (i > 0) {
-            const HitRaw pc = pv;
-            if (i > 1) pv = load_hit(a, h - 2 * hd);
-            decode_hit(B.align, pc, mpy, mpz, prow, psec);
-          }
-          const float2 gcur = gnx;
-          if (addg && i > 0) gnx = gmr[h - hd];
-          float b_mc[2], b_mp[2];
-          if (MAT)
-            step_rev_mat<FIELD>(G, T, &st[i & 1][0][lane], mpy, mpz, i == 0, pass == 0, row, side_sector(sec), m0,
-                                m1, b_p, b_L, b_chi, b_mc, b_mp);
-          else
-            step_rev<FIELD>(G, T, &st[i & 1][0][lane], mpy, mpz, i == 0, pass == 0, row, side_sector(sec), m0, m1,
-                            b_p, b_L, b_chi, b_mc, b_mp);
-          accumulate_meas_grad(a, pass, h, row, sec, b_mc[0] + pend0, b_mc[1] + pend1, gcur);
-          pend0 = b_mp[0];
-          pend1 = b_mp[1];
-          m0 = mpy;
-          m1 = mpz;
-          row = prow;
-          sec = psec;
+      while (hi > 0) {
+        int lo = 0;
+        const float4* sp = gs;  // this lane's float4 0 of step lo
+        int sp_pitch = kWarp;
+        if (taped) {
+          sp = tape_row0(a.tape, place, pitch, lane) + kSqrtRows * pass * place.y * pitch;
+          sp_pitch = pitch;
+        } else {
+          lo = (hi - 1) & ~(kCkptEvery - 1);
+          if (lo < steps)
+            recompute_segment<MAT, FIELD>(
+                a, T, B.align,
+                a.ck + ((int64_t)pass * a.ck_slots + (begin >> kCkptShift) + trk + (lo >> kCkptShift)) * kCkptFloats, gs,
+                h0, hd, lo, min(hi, steps) - lo, pass == 0);
+          __threadfence_block();  // the states just stored are read back by this thread's copies below
         }
-        // the inward pass starts from the outward result with the factor reset:
-        // b_p carries over, b_L does not
+        const int step_f4 = kSqrtRows * sp_pitch;
+        if (hi - 1 < steps) copy_rows<kSqrtRows>(&st[(hi - 1) & 1][0][lane], sp + (hi - 1 - lo) * step_f4, sp_pitch);
+        cp_async_commit();
+#pragma unroll 1
+        for (int i = hi - 1; i >= lo; --i) {
+          if (i > lo && i - 1 < steps)
+            copy_rows<kSqrtRows>(&st[(i - 1) & 1][0][lane], sp + (i - 1 - lo) * step_f4, sp_pitch);
+          cp_async_commit();
+          cp_async_wait<1>();
+          if (i < steps) {
+            const int h = h0 + hd * i;
+            float mpy = 0.0f, mpz = 0.0f;
+            int prow = 0, psec = 0;
+            if (i > 0) {
+              const HitRaw pc = pv;
+              if (i > 1) pv = load_hit(a, h - 2 * hd);
+              decode_hit(B.align, pc, mpy, mpz, prow, psec);
+            }
+            const float2 gcur = gnx;
+            if (addg && i > 0) gnx = gmr[h - hd];
+            float b_mc[2], b_mp[2];
+            if (MAT)
+              step_rev_mat<FIELD>(G, T, &st[i & 1][0][lane], mpy, mpz, i == 0, pass == 0, row, side_sector(sec), m0,
+                                  m1, b_p, b_L, b_chi, b_mc, b_mp);
+            else
+              step_rev<FIELD>(G, T, &st[i & 1][0][lane], mpy, mpz, i == 0, pass == 0, row, side_sector(sec), m0, m1,
+                              b_p, b_L, b_chi, b_mc, b_mp);
+            accumulate_meas_grad(a, pass, h, row, sec, b_mc[0] + pend0, b_mc[1] + pend1, gcur);
+            pend0 = b_mp[0];
+            pend1 = b_mp[1];
+            m0 = mpy;
+            m1 = mpz;
+            row = prow;
+            sec = psec;
+          }
+        }
+        hi = lo;
+        cp_async_wait<0>();
       }
-    } else if (a.grad_meas) {
-      const int b = a.off[trk];
+      // the inward pass starts from the outward result with the factor reset:
+      // b_p carries over, b_L does not
+    }
+    if (!have) continue;
+    if (!fitted && a.grad_meas) {
       const int end = a.off[trk + 1];
-      for (int h = b; h < end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
+      for (int h = begin; h < end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
     }
 #pragma unroll
     for (int c = 0; c < 5; ++c) a.grad_seeds[(int64_t)c * N + trk] = b_p[c];
   }
 }
-
-constexpr size_t kTapeReverseWarpSmem = (size_t)2 * kStateF4 * kWarp * sizeof(float4);
 
 // Persistent launch of a kernel with up to `warps` warps per block, `block_smem`
 // bytes of shared memory per block and `warp_smem` per warp.
@@ -1351,14 +1470,6 @@ cudaError_t launch_persistent(K kernel, Resident& r, int warps, size_t block_sme
   if (e != cudaSuccess) return e;
   kernel<<<w.blocks, w.warps * kWarp, block_smem + w.warps * warp_smem, s>>>(b);
   return cudaGetLastError();
-}
-
-template <int WARPS, int PHYS>
-cudaError_t launch_tape_backward_cfg(const BwdArgs& a, cudaStream_t s) {
-  static Resident g_rec, g_rev;
-  cudaError_t e = launch_persistent(recompute_kernel<PHYS>, g_rec, kRecomputeWarps, sizeof(BwdSmem), 0, a, s);
-  if (e != cudaSuccess) return e;
-  return launch_persistent(tape_reverse_kernel<WARPS, PHYS>, g_rev, WARPS, sizeof(BwdSmem), kTapeReverseWarpSmem, a, s);
 }
 
 // Blocks of the one-kernel backward resident at once.
@@ -1382,92 +1493,104 @@ cudaError_t launch_backward_cfg(const BwdArgs& a, cudaStream_t s) {
                            sizeof(BwdSmem), sizeof(BwdWarpBufsT<FORM ? kUDStateF4 : kStateF4>), a, s);
 }
 
-// Warps per block of a backward launch: the configured shape in a uniform
-// field without material; the other physics run in the 8-warp shape only.
-inline int backward_warps(int warps, int phys) { return phys ? 8 : warps; }
-
-// One-kernel fast backward (no material layers): FORM 0 or 1 in every
-// compiled block shape, uniform field (PHYS 0) or the field map (PHYS 2, 8
-// warps).
-template <int FORM>
-cudaError_t backward_store_form(int warps, int phys, int64_t& float4s) {
-  switch (phys) {
-    case 0: break;
-    case 2: return backward_store_cfg<8, 2, FORM>(float4s);
-    default: return cudaErrorInvalidValue;
-  }
+#if !TPCFIT_DET
+// The fast backward from checkpoints without material layers: in a uniform field
+// every compiled block shape, with the field map 8 warps.
+template <class F>
+cudaError_t for_backward_shape(int warps, int phys, F&& f) {
+  using std::integral_constant;
+  if (phys == 2) return f(integral_constant<int, 8>(), integral_constant<int, 2>());
+  if (phys != 0) return cudaErrorInvalidValue;
   switch (warps) {
-    case 4: return backward_store_cfg<4, 0, FORM>(float4s);
-    case 8: return backward_store_cfg<8, 0, FORM>(float4s);
-    case 10: return backward_store_cfg<10, 0, FORM>(float4s);
-    case 12: return backward_store_cfg<12, 0, FORM>(float4s);
+    case 4: return f(integral_constant<int, 4>(), integral_constant<int, 0>());
+    case 8: return f(integral_constant<int, 8>(), integral_constant<int, 0>());
+    case 10: return f(integral_constant<int, 10>(), integral_constant<int, 0>());
+    case 12: return f(integral_constant<int, 12>(), integral_constant<int, 0>());
     default: return cudaErrorInvalidValue;
   }
 }
 
-template <int FORM>
-cudaError_t launch_backward_form(const BwdArgs& a, int warps, cudaStream_t s) {
-  switch (a.phys) {
-    case 0: break;
-    case 2: return launch_backward_cfg<8, 2, FORM>(a, s);
-    default: return cudaErrorInvalidValue;
-  }
-  switch (warps) {
-    case 4: return launch_backward_cfg<4, 0, FORM>(a, s);
-    case 8: return launch_backward_cfg<8, 0, FORM>(a, s);
-    case 10: return launch_backward_cfg<10, 0, FORM>(a, s);
-    case 12: return launch_backward_cfg<12, 0, FORM>(a, s);
-    default: return cudaErrorInvalidValue;
-  }
+inline cudaError_t launch_checkpoint_backward(const BwdArgs& a, int warps, cudaStream_t s) {
+  return for_backward_shape(warps, a.phys, [&](auto w, auto p) {
+    return a.form == 1 ? launch_backward_cfg<w(), p(), 1>(a, s) : launch_backward_cfg<w(), p(), 0>(a, s);
+  });
 }
 
-// Segment store (float4 count) the backward needs for `warps` warps per block,
-// the physics bits phys (1: material layers, 2: the field map) and the factor
-// form (0: square root, 1: U-D).
+// The U-D reverse from the tape: 12 warps (168 registers) where there is work for
+// them (400,000 tracks, every state on the tape: 1.96 ms against 2.20 with 8, 212
+// registers), 8 otherwise (1,000 tracks: 304 us against 326).
+template <int PHYS>
+cudaError_t launch_tape_ud(const BwdArgs& a, cudaStream_t s) {
+  static Resident r1, r2;
+  if (a.tape_every == 1)
+    return launch_persistent(tape_reverse_ud_kernel<8, PHYS, 1>, r1, 8, sizeof(SmemTables), sizeof(TapeWarpUD<1>), a, s);
+  return launch_persistent(tape_reverse_ud_kernel<12, PHYS, 2>, r2, 12, sizeof(SmemTables), sizeof(TapeWarpUD<2>), a, s);
+}
+#endif
+
+constexpr int kTapeSqrtWarps = 8;
+template <int PHYS>
+Resident& tape_sqrt_resident() {
+  static Resident r;
+  return r;
+}
+template <int PHYS>
+cudaError_t tape_sqrt_store(int64_t& float4s) {
+  Resident& r = tape_sqrt_resident<PHYS>();
+  const cudaError_t e = resident_blocks(tape_reverse_kernel<kTapeSqrtWarps, PHYS>, kTapeSqrtWarps * kWarp,
+                                        sizeof(BwdSmem) + kTapeSqrtWarps * kTapeWarpSmemSqrt, r);
+  float4s = (int64_t)r.blocks * kTapeSqrtWarps * kCkptEvery * kStateF4 * kWarp;
+  return e;
+}
+template <int PHYS>
+cudaError_t launch_tape_sqrt(const BwdArgs& a, cudaStream_t s) {
+  return launch_persistent(tape_reverse_kernel<kTapeSqrtWarps, PHYS>, tape_sqrt_resident<PHYS>(), kTapeSqrtWarps,
+                           sizeof(BwdSmem), kTapeWarpSmemSqrt, a, s);
+}
+
+// Segment store (float4 count) the backward needs: in fast mode without material
+// (form 0 square root, 1 U-D) for the reverse from checkpoints in `warps`-warp
+// blocks, otherwise for the items that the tape has no room for.
 inline cudaError_t backward_store(int warps, int phys, int form, int64_t& float4s) {
-  if (form == 1) return backward_store_form<1>(warps, phys, float4s);
-  if (form == 0) return backward_store_form<0>(warps, phys, float4s);
-  return cudaErrorInvalidValue;
-}
-
-// The deterministic backward always, and the fast one with material layers,
-// replay the segments onto the tape (recompute_kernel + tape_reverse_kernel);
-// the fast backward without material recomputes into the segment store
-// (backward_kernel).
-inline cudaError_t launch_tape_backward(const BwdArgs& a, int warps, cudaStream_t s) {
-  switch (a.phys) {
-    case 0: break;
-    case 1: return launch_tape_backward_cfg<8, 1>(a, s);
-#if TPCFIT_DET
-    case 2: return launch_tape_backward_cfg<8, 2>(a, s);
+#if !TPCFIT_DET
+  if (!(phys & 1))
+    return for_backward_shape(warps, phys, [&](auto w, auto p) {
+      return form == 1 ? backward_store_cfg<w(), p(), 1>(float4s) : backward_store_cfg<w(), p(), 0>(float4s);
+    });
 #endif
-    case 3: return launch_tape_backward_cfg<8, 3>(a, s);
+  switch (phys) {
+#if TPCFIT_DET
+    case 0: return tape_sqrt_store<0>(float4s);
+    case 2: return tape_sqrt_store<2>(float4s);
+#endif
+    case 1: return tape_sqrt_store<1>(float4s);
+    case 3: return tape_sqrt_store<3>(float4s);
     default: return cudaErrorInvalidValue;
   }
-#if TPCFIT_DET
-  switch (warps) {
-    case 4: return launch_tape_backward_cfg<4, 0>(a, s);
-    case 8: return launch_tape_backward_cfg<8, 0>(a, s);
-    case 10: return launch_tape_backward_cfg<10, 0>(a, s);
-    case 12: return launch_tape_backward_cfg<12, 0>(a, s);
-    default: return cudaErrorInvalidValue;
-  }
-#else
-  (void)warps;
-  return cudaErrorInvalidValue;
-#endif
 }
 
 inline cudaError_t launch_backward(const BwdArgs& a, int warps, cudaStream_t s) {
   if (a.n_tracks <= 0) return cudaSuccess;
-  if (a.tape) return launch_tape_backward(a, warps, s);
-#if TPCFIT_DET
-  return cudaErrorInvalidValue;
-#else
-  if (a.form == 1) return launch_backward_form<1>(a, warps, s);
-  if (a.form == 0) return launch_backward_form<0>(a, warps, s);
-  return cudaErrorInvalidValue;
+#if !TPCFIT_DET
+  if (!(a.phys & 1)) {
+    // from the tape where the fit left one; the kernel from checkpoints then looks
+    // after the items that found no room on it
+    if (a.tape) {
+      const cudaError_t e = a.phys == 2 ? launch_tape_ud<2>(a, s) : launch_tape_ud<0>(a, s);
+      if (e != cudaSuccess) return e;
+    }
+    return launch_checkpoint_backward(a, warps, s);
+  }
 #endif
+  switch (a.phys) {
+#if TPCFIT_DET
+    case 0: return launch_tape_sqrt<0>(a, s);
+    case 2: return launch_tape_sqrt<2>(a, s);
+#endif
+    case 1: return launch_tape_sqrt<1>(a, s);
+    case 3: return launch_tape_sqrt<3>(a, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 }  // namespace TPCFIT_NS

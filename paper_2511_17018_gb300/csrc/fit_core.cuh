@@ -732,11 +732,57 @@ __device__ __forceinline__ void write_ckpt(const FitArgs& a, int pass, int begin
   for (int j = 0; j < kCkptFloats / 4; ++j) dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
 }
 
+// A work item's place on the tape (first row, or -1: it has no room), from the
+// counter of the rows handed out; n: clusters of its longest track.
+template <int FORM>
+__device__ __forceinline__ int take_tape(const FitArgs& a, int64_t item, int n) {
+  int first = 0;
+  if ((threadIdx.x & 31) == 0) {
+    if (n > 0) {
+      const unsigned long long need = (unsigned long long)tape_rows(FORM == 1, n, a.tape_every);
+      const unsigned long long at = atomicAdd(reinterpret_cast<unsigned long long*>(a.work + kWorkTape), need);
+      // (the bound on n keeps offsets within an item's part in 32 bits)
+      first = n < (1 << 21) && at + need <= (unsigned long long)a.tape_rows ? (int)at : -1;
+      if (first < 0) atomicAdd(a.work + kWorkMissing, 1u);
+    }
+    a.tape_item[item] = make_int2(first, n);
+  }
+  return __shfl_sync(0xffffffffu, first, 0);
+}
+
+// A state's rows of the tape (dst: the lane's float4 of the first one; pitch:
+// tracks of the item).  Written once and read once by a later kernel: streaming
+// stores, so that the clusters stay in L2 for the inward pass (400,000 tracks,
+// every state: 1.54 ms against 1.80 with plain stores).
+template <int FORM>
+__device__ __forceinline__ void write_tape(float4* dst, int pitch, const TrackState& S) {
+  constexpr int N = FORM == 1 ? kUDRows : kSqrtRows;
+  float v[4 * N];
+#pragma unroll
+  for (int c = 0; c < 5; ++c) v[c] = S.p[c];
+  if (FORM == 1) {
+#pragma unroll
+    for (int e = 0; e < 10; ++e) v[5 + e] = S.u[e];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) v[15 + c] = S.d[c];
+  } else {
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+#pragma unroll
+      for (int c = 0; c < 5; ++c) v[5 + 5 * i + c] = S.L[i][c];
+    v[4 * N - 2] = S.x;
+    v[4 * N - 1] = __int_as_float(S.sec);
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) __stcs(dst + j * pitch, make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
+}
+
 // PHYS: bit 0 the material layers, bit 1 the field map (compile-time variants,
 // so that the plain fit carries neither).  FORM: the covariance's factor, 0
 // the square-root factor with Potter's updates (the canonical sequence of the
 // deterministic mode), 1 U-D with Bierman's (fast mode, no material layers).
-template <int RPS, int WARPS, int MINB, bool RECORD, bool FRAMES, int PHYS, int FORM = 0>
+// RECORD: 0 nothing, 1 checkpoints, 2 the tape.
+template <int RPS, int WARPS, int MINB, int RECORD, bool FRAMES, int PHYS, int FORM = 0>
 __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_constant__ FitArgs a) {
   const GeoRef& G = TPCFIT_GEO(a);
   constexpr bool MAT = (PHYS & 1) != 0;
@@ -804,6 +850,17 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
       for (int c = 0; c < 5; ++c) S.p[c] = __ldg(a.seeds + (int64_t)c * a.n_tracks + trk);
       if (!(fabsf(S.p[2]) < G.max_snp)) status = 2;
     }
+    bool on_tape = false;
+    float4* tape = nullptr;  // this lane's float4 of the item's first row
+    int tape_n = 0;
+    if (RECORD == 2) {
+      tape_n = status == 0 ? n : 0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) tape_n = max(tape_n, __shfl_xor_sync(0xffffffffu, tape_n, o));
+      const int at = take_tape<FORM>(a, item, tape_n);
+      on_tape = at >= 0;
+      tape = a.tape + (int64_t)at * a.item_tracks + lane;
+    }
 
     // ---- two passes: outward (dir +1 from hit 0) and inward (dir -1 from `last`)
 #pragma unroll 1
@@ -812,6 +869,11 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
       const int my_first = begin + (pass == 0 ? 0 : last);
       const int my_count = (status == 0) ? (pass == 0 ? n : last + 1) : 0;
       bool go = status == 0;
+      // the pass's first state on the tape, from the item's row 0
+      int tape_pass = 0;
+      if (RECORD == 2)
+        tape_pass = a.item_tracks * (FORM == 1 ? tape_n + kUDRows * (pass * (int)tape_states(tape_n, a.tape_every))
+                                               : kSqrtRows * (pass * tape_n));
       if (go) {
         if (FORM == 1) {
 #pragma unroll
@@ -861,7 +923,19 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
           const float m0 = st.y[buf][lane][k] - d.x;
           const float m1 = st.z[buf][lane][k] - d.y;
           const int sec18 = side_sector(sec);
-          if (RECORD && (i & (kCkptEvery - 1)) == 0) write_ckpt<FORM>(a, pass, begin, trk, i >> kCkptShift, S);
+          if (RECORD == 2 && on_tape) {
+            if (FORM == 1) {
+              if (pass == 0)
+                __stcs(tape + i * a.item_tracks, make_float4(m0, m1, T.row_x[row], __int_as_float(rsv)));
+              const int skip = a.tape_every - 1;  // 0 or 1
+              if ((i & skip) == 0)
+                write_tape<1>(tape + tape_pass + (i >> skip) * (kUDRows * a.item_tracks), a.item_tracks, S);
+            } else {
+              write_tape<0>(tape + tape_pass + i * (kSqrtRows * a.item_tracks), a.item_tracks, S);
+            }
+          } else if (RECORD && (i & (kCkptEvery - 1)) == 0) {
+            write_ckpt<FORM>(a, pass, begin, trk, i >> kCkptShift, S);
+          }
           if (i == 0) {
             // first cluster of the pass: the state sits on its row already; the
             // outward pass turns the seed's (y, z) into residuals
@@ -970,7 +1044,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
 }
 
 #ifndef __CUDACC_RTC__
-template <int RPS, int WARPS, int MINB, bool RECORD, bool FRAMES, int PHYS, int FORM>
+template <int RPS, int WARPS, int MINB, int RECORD, bool FRAMES, int PHYS, int FORM>
 cudaError_t launch_cfg(const FitArgs& a, cudaStream_t s) {
   constexpr int kThreads = WARPS * 32;
   const size_t smem = sizeof(BlockSmem) + WARPS * sizeof(WarpStage<RPS>);
@@ -981,7 +1055,7 @@ cudaError_t launch_cfg(const FitArgs& a, cudaStream_t s) {
   const WorkShape w = work_shape(a.n_tracks, r.blocks, WARPS, r.sms);
   FitArgs b = a;
   b.item_tracks = w.tracks;
-  if (needs_work_counter(w)) e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
+  e = clear_work(a.work, RECORD == 2, needs_work_counter(w), s);
   if (e != cudaSuccess) return e;
   kernel<<<w.blocks, w.warps * kWarp, sizeof(BlockSmem) + w.warps * sizeof(WarpStage<RPS>), s>>>(b);
   return cudaGetLastError();
@@ -990,7 +1064,7 @@ cudaError_t launch_cfg(const FitArgs& a, cudaStream_t s) {
 // Supported (rows per stage, warps per block) shapes; the shared-memory budget
 // (alignment table + double buffer) decides how many blocks fit on an SM.
 // With material or a field map the fit runs at (4, 24).
-template <bool RECORD, bool FRAMES, int FORM>
+template <int RECORD, bool FRAMES, int FORM>
 inline cudaError_t launch_rec(const FitArgs& a, int rps, int warps, cudaStream_t s) {
   const int phys = (a.mat ? 1 : 0) | (a.field ? 2 : 0);
   if (FORM == 0) {
@@ -999,6 +1073,10 @@ inline cudaError_t launch_rec(const FitArgs& a, int rps, int warps, cudaStream_t
   } else if (phys & 1) {
     return cudaErrorInvalidValue;
   }
+#if !TPCFIT_DET
+  // the fast fit in square-root form is taped with material layers only
+  if constexpr (FORM == 0 && RECORD == 2) return cudaErrorInvalidValue;
+#endif
   if (phys == 2) return launch_cfg<4, 24, fit_min_blocks(4, 24), RECORD, FRAMES, 2, FORM>(a, s);
   if (rps == 4 && warps == 8) return launch_cfg<4, 8, fit_min_blocks(4, 8), RECORD, FRAMES, 0, FORM>(a, s);
   if (rps == 4 && warps == 12) return launch_cfg<4, 12, fit_min_blocks(4, 12), RECORD, FRAMES, 0, FORM>(a, s);
@@ -1011,9 +1089,9 @@ inline cudaError_t launch_rec(const FitArgs& a, int rps, int warps, cudaStream_t
 
 template <int FORM>
 inline cudaError_t launch_form(const FitArgs& a, int rps, int warps, cudaStream_t s) {
-  if (a.frame_base)
-    return a.ck ? launch_rec<true, true, FORM>(a, rps, warps, s) : launch_rec<false, true, FORM>(a, rps, warps, s);
-  return a.ck ? launch_rec<true, false, FORM>(a, rps, warps, s) : launch_rec<false, false, FORM>(a, rps, warps, s);
+  if (a.frame_base) return launch_rec<0, true, FORM>(a, rps, warps, s);  // batched frames are not recorded
+  if (a.tape) return launch_rec<2, false, FORM>(a, rps, warps, s);
+  return a.ck ? launch_rec<1, false, FORM>(a, rps, warps, s) : launch_rec<0, false, FORM>(a, rps, warps, s);
 }
 
 // One lane per track.  FORM 1 (U-D) in fast mode without material layers,

@@ -71,17 +71,26 @@ inline WorkShape work_shape(int64_t n_tracks, int resident, int max_warps, int s
 }
 inline bool needs_work_counter(const WorkShape& w) { return w.items > w.blocks * w.warps; }
 
+// Tracks per work item alone (what the tape's layout depends on).
+inline int32_t item_tracks(int64_t n_tracks, int sms) { return work_shape(n_tracks, 1, 1, sms).tracks; }
+// Clear a launch's counters: the tape's (with the work item counter), the work
+// item counter alone, or nothing.
+inline cudaError_t clear_work(unsigned int* work, bool tape, bool counter, cudaStream_t s) {
+  if (tape) return cudaMemsetAsync(work, 0, 4 * sizeof(unsigned int), s);
+  if (counter) return cudaMemsetAsync(work, 0, sizeof(unsigned int), s);
+  return cudaSuccess;
+}
+
 // ---- kernel launchers, one per module
 cudaError_t launch_fit_fast(const FitArgs& a, int lanes_per_track, int rows_per_stage, int warps, cudaStream_t s);
 cudaError_t launch_fit_det(const FitArgs& a, int lanes_per_track, int rows_per_stage, int warps, cudaStream_t s);
 cudaError_t launch_backward_fast(const BwdArgs& a, int warps, cudaStream_t s);
 cudaError_t launch_backward_det(const BwdArgs& a, int warps, cudaStream_t s);
-// float4 elements of the segment store a fast backward launch without material
-// with `warps`, the physics bits phys and the factor form (0 square root, 1 U-D)
-// needs
+// float4 elements of the segment store a backward launch needs (`warps`: of the
+// reverse from checkpoints; the physics bits phys; the factor form, 0 square root,
+// 1 U-D)
 cudaError_t backward_store_fast(int warps, int phys, int form, int64_t& float4s);
-// float4 elements of the backward's tape for n_tracks tracks
-int64_t backward_tape_float4s(int64_t n_tracks);
+cudaError_t backward_store_det(int warps, int phys, int form, int64_t& float4s);
 // the two-filter smoother of a recorded fit, and its segment store (float4s)
 cudaError_t launch_smooth_fast(const SmoothArgs& a, cudaStream_t s);
 cudaError_t launch_smooth_det(const SmoothArgs& a, cudaStream_t s);
@@ -112,7 +121,8 @@ const char* rtc_log();
 std::string rtc_fit_source(const GeoConst& g, bool det);
 // NVRTC only (no device needed): the CUBIN of a variant, stored in cache_dir
 // when given.
-tpcfit_status rtc_build(const GeoConst& g, bool det, int rps, int warps, bool record, bool frames,
+// record: 0 nothing, 1 checkpoints, 2 the tape.
+tpcfit_status rtc_build(const GeoConst& g, bool det, int rps, int warps, int record, bool frames,
                         const char* cache_dir);
 // Compile (once per source and variant) and launch the fit specialised for g.
 tpcfit_status rtc_launch_fit(const GeoConst& g, bool det, int rps, int warps, const FitArgs& a, const char* cache_dir,

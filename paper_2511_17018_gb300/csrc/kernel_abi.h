@@ -58,6 +58,29 @@ struct GeoConst {
   float f_r, f_z;             // c_r / 250^2, c_z / 250^2 [1/cm^2]
 };
 
+// The tape of a recorded fit: states of both passes, written by the fit and read by
+// the adjoint.  A work item of T tracks has rows of T float4 there, one float4 a
+// track, so that a warp's access to a row is contiguous.  With n the clusters of
+// the item's longest track, in this order:
+//   U-D form: n rows, row i the cluster i of each track (measured y, z with the
+//     alignment taken off, the row's x, row << 6 | sector); then for the outward
+//     and for the inward pass 5 rows (p 5, u 10, d 5) for the state before every
+//     `every`-th step;
+//   square-root form: for each pass 8 rows (p 5, L 25, x, sector) a step.
+// tape_item[item] = {first row, n}; an item that found no room (first < 0)
+// leaves checkpoints instead.
+// The launch's counters (FitArgs::work): words 0 the next work item, 1 the items
+// without a place on the tape, 2-3 (64 bits) the rows handed out.
+constexpr int kUDRows = 5;
+constexpr int kSqrtRows = 8;
+constexpr int kWorkMissing = 1;
+constexpr int kWorkTape = 2;
+// States of a pass of n steps, and rows of an item.
+__host__ __device__ constexpr int64_t tape_states(int64_t n, int every) { return (n + every - 1) / every; }
+__host__ __device__ constexpr int64_t tape_rows(bool ud, int64_t n, int every) {
+  return ud ? n + 2 * kUDRows * tape_states(n, every) : 2 * kSqrtRows * n;
+}
+
 // Arguments of one fit launch.
 struct FitArgs {
   GeoConst geo;                // the time frame's constants
@@ -80,6 +103,11 @@ struct FitArgs {
   float* ck;                   // [2][ck_slots][32] filter state before every kCkptEvery-th step of each pass
   int32_t* ck_last;            // [n_tracks] index of the last cluster of the outward pass
   int64_t ck_slots;            // slots per pass: n_hits / kCkptEvery + n_tracks + 1
+  // or the tape (null = checkpoints)
+  float4* tape;
+  int2* tape_item;             // [items] place of an item's rows on the tape
+  int64_t tape_rows;           // rows of item_tracks float4 the tape holds
+  int32_t tape_every;          // U-D form: steps from one state to the next (1 or 2)
   // several time frames in one launch (frame_base = null: one frame)
   const int64_t* frame_base;   // [n_frames + 1] first track of each frame
   int32_t n_frames;
@@ -113,7 +141,9 @@ struct BwdArgs {
   float* grad_align_atomic;    // [36][152][2] accumulated with atomics, or null
   unsigned int* work;
   float4* seg;                 // segment store: [resident warps][kCkptEvery][8][32] float4
-  float4* tape;                // or the tape: [2][n_hits][8] float4, the state before every step (null: segment store)
+  const float4* tape;          // the recorded fit's tape, or null (checkpoints only)
+  const int2* tape_item;       // [items] (null without a tape)
+  int32_t tape_every;
   int32_t phys;                // physics of the recorded fit: bit 1 material layers, bit 2 the field map
   int32_t form;                // factor the fast one-kernel backward recomputes in: 0 square root (L), 1 U-D
   int32_t ck_form;             // factor the checkpoints hold: 0 L, 1 U-D (u, d)
@@ -142,7 +172,10 @@ struct SmoothArgs {
   float* state_cov;            // [n_hits][15] its covariance (packed)
   unsigned int* work;
   float4* seg;                 // segment store, as for the adjoint
-  int32_t ck_form;             // factor the checkpoints hold: 0 L, 1 U-D (u, d)
+  int32_t ck_form;             // factor the checkpoints or the tape hold: 0 L, 1 U-D (u, d)
+  const float4* tape;          // the recorded fit's tape, or null (checkpoints only)
+  const int2* tape_item;       // [items] (null without a tape)
+  int32_t tape_every;
   int32_t mat;                 // material layers on (the recorded fit had them)
   int32_t item_tracks;         // tracks per work item (set by the launcher)
 };

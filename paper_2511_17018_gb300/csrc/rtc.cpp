@@ -240,11 +240,11 @@ struct Variant {
   std::string src, expr, key;
 };
 
-Variant variant(const GeoConst& g, bool det, int rps, int warps, bool record, bool frames, int form) {
+Variant variant(const GeoConst& g, bool det, int rps, int warps, int record, bool frames, int form) {
   Variant v;
   v.src = rtc_fit_source(g, det);
   v.expr = "tpcfit::rtc::fit_kernel<" + std::to_string(rps) + ", " + std::to_string(warps) + ", " +
-           std::to_string(fit_min_blocks(rps, warps)) + ", " + (record ? "true" : "false") + ", " +
+           std::to_string(fit_min_blocks(rps, warps)) + ", " + std::to_string(record) + ", " +
            (frames ? "true" : "false") + ", " + std::to_string((g.mat ? 1 : 0) | (g.field ? 2 : 0)) + ", " +
            std::to_string(form) + ">";
   std::string opt;
@@ -286,7 +286,7 @@ tpcfit_status cubin_of(const Variant& v, bool det, const char* cache_dir, std::v
 
 }  // namespace
 
-tpcfit_status rtc_build(const GeoConst& g, bool det, int rps, int warps, bool record, bool frames,
+tpcfit_status rtc_build(const GeoConst& g, bool det, int rps, int warps, int record, bool frames,
                         const char* cache_dir) {
   // the library's default factor: U-D in fast mode without material layers
   const Variant v = variant(g, det, rps, warps, record, frames, (!det && !g.mat) ? 1 : 0);
@@ -298,7 +298,7 @@ tpcfit_status rtc_build(const GeoConst& g, bool det, int rps, int warps, bool re
 tpcfit_status rtc_launch_fit(const GeoConst& g, bool det, int rps, int warps, const FitArgs& a, const char* cache_dir,
                              cudaStream_t s) {
   if (a.n_tracks <= 0) return TPCFIT_OK;
-  const Variant v = variant(g, det, rps, warps, a.ck != nullptr, a.frame_base != nullptr,
+  const Variant v = variant(g, det, rps, warps, a.tape ? 2 : (a.ck ? 1 : 0), a.frame_base != nullptr,
                             (!det && !g.mat && a.form == 1) ? 1 : 0);
   const std::string& key = v.key;
   Compiled* c = nullptr;
@@ -352,8 +352,7 @@ tpcfit_status rtc_launch_fit(const GeoConst& g, bool det, int rps, int warps, co
   const WorkShape w = work_shape(a.n_tracks, r.blocks, warps, r.sms);
   FitArgs args = a;
   args.item_tracks = w.tracks;
-  if (needs_work_counter(w)) e = cudaMemsetAsync(a.work, 0, sizeof(unsigned int), s);
-  if (e != cudaSuccess) return TPCFIT_ECUDA;
+  if (clear_work(a.work, a.tape != nullptr, needs_work_counter(w), s) != cudaSuccess) return TPCFIT_ECUDA;
   void* params[] = {&args};
   e = cudaLaunchKernel(fn, dim3(w.blocks), dim3(w.warps * kWarp), params,
                        (size_t)kFitBlockSmemBytes + (size_t)w.warps * fit_warp_stage_bytes(rps), s);

@@ -227,6 +227,66 @@ __device__ __forceinline__ void write_nan_clusters(const SmoothArgs& a, int h0, 
   }
 }
 
+// The state before step i of a pass as the recorded fit left it: from the tape or
+// from its checkpoint (i a multiple of kCkptEvery).  Copied asynchronously into
+// the warp's lane-interleaved checkpoint buffer, as one commit group; a U-D
+// state's x and sector are those of the cluster before the step.
+struct RecordedPass {
+  const float4* src;       // tape: this lane's float4 of the pass's first state; checkpoints: the first one
+  const float4* cluster;   // U-D tape: this lane's cluster of step 0
+  int pitch;               // tape: tracks of the item; 0: checkpoints
+  int cluster_step;
+};
+
+__device__ __forceinline__ RecordedPass recorded_pass(const SmoothArgs& a, int2 place, int pass, int lane, int begin,
+                                                      int trk, int steps) {
+  RecordedPass r;
+  r.cluster = nullptr;
+  r.cluster_step = 0;
+  if (a.tape_item && place.x >= 0) {
+    r.pitch = a.item_tracks;
+    const float4* row0 = tape_row0(a.tape, place, r.pitch, lane);
+    if (a.ck_form == 1) {
+      r.src = row0 + (place.y + kUDRows * pass * (int)tape_states(place.y, a.tape_every)) * r.pitch;
+      r.cluster = row0 + (pass == 0 ? 0 : steps - 1) * r.pitch;
+      r.cluster_step = pass == 0 ? r.pitch : -r.pitch;
+    } else {
+      r.src = row0 + kSqrtRows * pass * place.y * r.pitch;
+    }
+  } else {
+    r.pitch = 0;
+    r.src = reinterpret_cast<const float4*>(a.ck + ((int64_t)pass * a.ck_slots + (begin >> kCkptShift) + trk) * kCkptFloats);
+  }
+  return r;
+}
+
+__device__ __forceinline__ void fetch_recorded(float4* sdst, const SmoothArgs& a, const RecordedPass& r, int i) {
+  if (r.pitch == 0) {
+    fetch_ckpt(sdst, reinterpret_cast<const float*>(r.src) + (int64_t)(i >> kCkptShift) * kCkptFloats);
+    return;
+  }
+  if (a.ck_form == 1) {
+    copy_rows<kUDRows>(sdst, r.src + i / a.tape_every * (kUDRows * r.pitch), r.pitch);
+    if (i > 0) cp_async16(sdst + kUDRows * kWarp, r.cluster + (i - 1) * r.cluster_step);
+  } else {
+    copy_rows<kSqrtRows>(sdst, r.src + i * (kSqrtRows * r.pitch), r.pitch);
+  }
+  cp_async_commit();
+}
+
+// The fetched state (after a wait), as the square-root factor.
+__device__ __forceinline__ void read_recorded(const float4* src, const SmoothArgs& a, const RecordedPass& r, int i,
+                                              StepState& S) {
+  read_state(src, S);
+  if (a.ck_form != 1) return;
+  sqrt_from_ud_ckpt(S);
+  if (r.pitch != 0 && i > 0) {
+    const float4 c = src[kUDRows * kWarp];
+    S.x = c.z;
+    S.sec = side_sector(__float_as_int(c.w) & 63);
+  }
+}
+
 // Shared memory of a smoother block: the tables, the alignment table and,
 // per warp, a double buffer for the inward states and a checkpoint buffer.
 template <int WARPS>
@@ -263,18 +323,22 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
     }
     const int last = a.ck_last[trk];
     write_nan_clusters(a, begin + last + 1, end);  // clusters the outward pass did not reach
-    const int64_t slot0 = (begin >> kCkptShift) + trk;
-    // outward filter: from its first checkpoint (the seed, factor L0)
+    const int2 place = a.tape_item ? a.tape_item[item] : make_int2(-1, 0);
+    // outward filter: from its first state (the seed, factor L0)
     StepState O;
-    load_ckpt(a.ck + slot0 * kCkptFloats, O);
-    if (a.ck_form == 1) sqrt_from_ud_ckpt(O);
+    {
+      const RecordedPass out = recorded_pass(a, place, 0, lane, begin, trk, last + 1);
+      fetch_recorded(&W.ck[0][lane], a, out, 0);
+      cp_async_wait<0>();
+      read_recorded(&W.ck[0][lane], a, out, 0, O);
+    }
     float omy = 0.0f, omz = 0.0f;  // measurement O's residuals refer to (none for the seed)
     // inward segments, last first: inward step j is cluster last - j
     const int steps = last + 1;
     const int nseg = (steps + kCkptEvery - 1) / kCkptEvery;
-    const float* ckp = a.ck + ((int64_t)a.ck_slots + slot0) * kCkptFloats;
+    const RecordedPass in = recorded_pass(a, place, 1, lane, begin, trk, last + 1);
     const int h_last = begin + last;
-    fetch_ckpt(&W.ck[0][lane], ckp + (int64_t)(nseg - 1) * kCkptFloats);
+    fetch_recorded(&W.ck[0][lane], a, in, (nseg - 1) * kCkptEvery);
 #pragma unroll 1
     for (int s = nseg - 1; s >= 0; --s) {
       const int j0 = s * kCkptEvery;
@@ -287,8 +351,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
         decode_hit(B.align, load_hit(a.y, a.z, a.rowsec, h_last - (j0 - 1)), my, mz, row, sec);
       }
       cp_async_wait<0>();
-      read_state(&W.ck[0][lane], S);
-      if (a.ck_form == 1) sqrt_from_ud_ckpt(S);
+      read_recorded(&W.ck[0][lane], a, in, j0, S);
       // level 1: the inward segment, storing the state before each step
 #pragma unroll 1
       for (int kk = 0; kk < cnt; ++kk) {
@@ -302,7 +365,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
         step_fwd<MAT, 2>(G, T, S, my, mz, j == 0, false, row, side_sector(sec), m0, m1);
       }
       __threadfence_block();  // the states just stored are read back by this thread's copies below
-      if (s > 0) fetch_ckpt(&W.ck[0][lane], ckp + (int64_t)(s - 1) * kCkptFloats);
+      if (s > 0) fetch_recorded(&W.ck[0][lane], a, in, (s - 1) * kCkptEvery);
       fetch_state(&W.st[(cnt - 1) & 1][0][lane], gs + (cnt - 1) * (kStateF4 * kWarp));
       // consume in reverse: cluster c = last - j ascending
 #pragma unroll 1

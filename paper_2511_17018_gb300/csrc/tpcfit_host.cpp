@@ -72,6 +72,7 @@ constexpr int kHostChunksMax = 8;
 
 struct tpcfit_handle {
   int device = 0;
+  int sms = 0;
   GeoConst geo{};
   int deterministic = 0;
   int lanes_per_track = 1;
@@ -97,7 +98,7 @@ struct tpcfit_handle {
   cudaEvent_t pipe_free[2] = {nullptr, nullptr};
   // tpcfit_fit_host: one event per chunk copied
   cudaEvent_t chunk_in[kHostChunksMax] = {};
-  // adjoint: checkpoints of the last recorded fit
+  // adjoint: checkpoints or tape of the last recorded fit
   int record = 0;
   int bwd_warps = 8;
   int bwd_form = 1;            // factor of the fast one-kernel backward: 1 U-D, 0 square root
@@ -117,8 +118,12 @@ struct tpcfit_handle {
   // adjoint scratch: per-cluster gradients and the key sort
   float4* d_seg = nullptr;     // the segment store of the backward (fast mode) and the smoother
   int64_t seg_cap = 0;         // float4 elements
-  float4* d_tape = nullptr;    // the backward's tape: the state before every step of both passes
+  float4* d_tape = nullptr;    // the recorded fit's tape: the state before every step of both passes
   int64_t tape_cap = 0;        // float4 elements
+  int2* d_tape_item = nullptr; // places of the work items on it
+  int64_t tape_item_cap = 0;
+  bool rec_tape = false;       // the recorded fit wrote the tape, with every
+  int rec_every = 1;           //   rec_every-th state (U-D form)
   float* d_gm = nullptr;
   int64_t gm_cap = 0;          // floats
   unsigned char* d_keys = nullptr;
@@ -163,6 +168,48 @@ tpcfit_status ensure_pipe(tpcfit_handle* h) {
   for (int i = 0; i < kHostChunksMax && e == cudaSuccess; ++i)
     e = cudaEventCreateWithFlags(&h->chunk_in[i], cudaEventDisableTiming);
   return from_cuda(e);
+}
+
+// Room for the tape of a recorded fit (kernel_abi.h) and its shape; without one
+// (a.tape null) the fit leaves checkpoints: another form of fit, no memory, or a
+// tape of more than half of what is free.
+void ensure_tape(tpcfit_handle* h, FitArgs& a) {
+  const bool ud = a.form == 1;
+  if (h->lanes_per_track != 1 || !(h->deterministic || a.mat || ud)) return;
+  const int64_t T = item_tracks(a.n_tracks, h->sms);
+  const int64_t items = ((int64_t)a.n_tracks + T - 1) / T;
+  // every state as long as the reverse's warps are all resident at once, then
+  // every second one (100,000 tracks, fit + reverse: 400 + 525 us with every
+  // state, 305 + 600 with every second one)
+  const int every = ud && items > 8 * (int64_t)h->sms ? 2 : 1;
+  // items of tracks sorted by length: an item's longest track is no longer than
+  // the mean track of the item before it, so all items together take at most
+  // n_hits / T steps a pass and the longest track's (the ordering tells lengths
+  // below 255 apart).  Unsorted: full tracks.
+  const int64_t rows = h->sort_by_length ? tape_rows(ud, a.n_hits / T + 256, every) + items * 2 * kUDRows
+                                         : items * tape_rows(ud, kMaxRows, every);
+  if (rows > INT32_MAX) return;
+  const int64_t need = rows * T;
+  if (need > h->tape_cap) {
+    size_t avail = 0, total = 0;
+    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    if (sizeof(float4) * (uint64_t)need > (avail + sizeof(float4) * (uint64_t)h->tape_cap) / 2) return;
+    if (grow(h->d_tape, h->tape_cap, need) != TPCFIT_OK) {
+      cudaGetLastError();
+      return;
+    }
+  }
+  if (grow(h->d_tape_item, h->tape_item_cap, items) != TPCFIT_OK) {
+    cudaGetLastError();
+    return;
+  }
+  a.tape = h->d_tape;
+  a.tape_item = h->d_tape_item;
+  a.tape_rows = rows;
+  a.tape_every = every;
 }
 
 tpcfit_status ensure_perm(tpcfit_handle* h, int64_t n) {
@@ -220,6 +267,7 @@ tpcfit_status tpcfit_create(const tpcfit_geometry* geometry, double bz_tesla, tp
     return TPCFIT_EINVAL;
   }
   cudaError_t e = cudaGetDevice(&h->device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_align, sizeof(float) * kAlignFloats);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_err, sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMalloc(&h->d_work, sizeof(unsigned int) * 64);
@@ -257,6 +305,7 @@ void tpcfit_destroy(tpcfit_handle* h) {
   if (h->d_gm) cudaFree(h->d_gm);
   if (h->d_seg) cudaFree(h->d_seg);
   if (h->d_tape) cudaFree(h->d_tape);
+  if (h->d_tape_item) cudaFree(h->d_tape_item);
   if (h->d_keys) cudaFree(h->d_keys);
   if (h->d_frame_scratch) cudaFree(h->d_frame_scratch);
   if (h->d_reject) cudaFree(h->d_reject);
@@ -338,6 +387,9 @@ tpcfit_status tpcfit_fit(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
     a.ck_last = h->d_ck_last;
     a.ck_slots = slots;
     h->ck_slots = slots;
+    ensure_tape(h, a);
+    h->rec_tape = a.tape != nullptr;
+    h->rec_every = a.tape_every;
   }
   if (h->sort_by_length) {
     st = ensure_perm(h, n_tracks);
@@ -497,7 +549,9 @@ tpcfit_status tpcfit_rtc_build(const tpcfit_geometry* geometry, double bz_tesla,
   GeoConst g{};
   if (!geometry || !build_geo(geometry, bz_tesla, g)) return TPCFIT_EINVAL;
   if (!fit_shape_supported(1, rows_per_stage, warps_per_block)) return TPCFIT_EINVAL;
-  return rtc_build(g, deterministic != 0, rows_per_stage, warps_per_block, record != 0, frames != 0, cache_dir);
+  // a recorded fit of the library's default factor leaves the tape
+  return rtc_build(g, deterministic != 0, rows_per_stage, warps_per_block, record != 0 && frames == 0 ? 2 : 0,
+                   frames != 0, cache_dir);
 }
 
 int tpcfit_rtc_available(void) { return rtc_available() ? 1 : 0; }
@@ -546,32 +600,27 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
   b.phys = (h->geo.mat ? 1 : 0) | (h->geo.field ? 2 : 0);
   b.ck_form = h->rec_form;
   cudaError_t e = cudaSuccess;
-  if (h->deterministic || h->geo.mat) {
-    // where the forward step is expensive (no FMA; the material folding) the
-    // backward replays the segments in a kernel of its own at the fit's
-    // occupancy onto a tape (the state before every step of both passes, 152
-    // steps per 32-track work item) and reverses from it; measured on 400k
-    // tracks: deterministic 8.0 ms against 9.5 ms, material 7.0 against 9.4
-    st = grow(h->d_tape, h->tape_cap, backward_tape_float4s(n_tracks));
-    if (st != TPCFIT_OK) return st;
+  // the square-root reverse hands each segment's factor adjoint to the segment
+  // before it, which holds only if its recomputation reproduces the recorded
+  // factor: after a U-D fit only the U-D reverse applies (the U-D factorisation of
+  // a covariance is unique)
+  const bool sqrt_only = h->deterministic || h->geo.mat;
+  if (!sqrt_only && h->bwd_form == 0 && h->rec_form == 1) return TPCFIT_ESTATE;
+  b.form = sqrt_only ? 0 : h->bwd_form;
+  if (h->rec_tape) {
     b.tape = h->d_tape;
-  } else {
-    // otherwise one kernel recomputes each segment into a per-warp segment
-    // store that stays in L2 until the reverse reads it back (square-root
-    // factor: 4.7 ms against 5.6 ms with the tape)
-    int64_t need = 0;
-    // the square-root reverse hands each segment's factor adjoint to the
-    // segment before it, which holds only if its recomputation reproduces the
-    // recorded factor: after a U-D fit only the U-D reverse applies (the U-D
-    // factorisation of a covariance is unique)
-    if (h->bwd_form == 0 && h->rec_form == 1) return TPCFIT_ESTATE;
-    b.form = h->bwd_form;
-    e = backward_store_fast(h->bwd_warps, b.phys, b.form, need);
-    if (e != cudaSuccess) return from_cuda(e);
-    st = grow(h->d_seg, h->seg_cap, need);
-    if (st != TPCFIT_OK) return st;
-    b.seg = h->d_seg;
+    b.tape_item = h->d_tape_item;
+    b.tape_every = h->rec_every;
   }
+  // from checkpoints, one kernel recomputes each segment into a per-warp segment
+  // store that stays in L2 until the reverse reads it back
+  int64_t need = 0;
+  e = h->deterministic ? backward_store_det(h->bwd_warps, b.phys, b.form, need)
+                       : backward_store_fast(h->bwd_warps, b.phys, b.form, need);
+  if (e != cudaSuccess) return from_cuda(e);
+  st = grow(h->d_seg, h->seg_cap, need);
+  if (st != TPCFIT_OK) return st;
+  b.seg = h->d_seg;
   if (!h->deterministic) {
     // fast: atomics straight into the alignment gradient
     b.grad_meas = grad_meas;
@@ -652,6 +701,11 @@ tpcfit_status run_smooth(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
   a.work = h->d_work;
   a.mat = h->geo.mat;
   a.ck_form = h->rec_form;
+  if (h->rec_tape) {
+    a.tape = h->d_tape;
+    a.tape_item = h->d_tape_item;
+    a.tape_every = h->rec_every;
+  }
   int64_t need = 0;
   cudaError_t e = h->deterministic ? smooth_store_det(need) : smooth_store_fast(need);
   if (e != cudaSuccess) return from_cuda(e);

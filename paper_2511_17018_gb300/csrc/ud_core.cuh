@@ -329,10 +329,10 @@ __device__ __forceinline__ void ud_state_from(const StepState& C, bool ud_ck, UD
 // that fails here on a rounding difference leaves the state unpropagated.
 template <int FIELD = 0>
 __device__ __forceinline__ void step_fwd_ud(const GeoRef& G, const SmemTables& T, UDState& S, float& my, float& mz,
-                                            bool first, bool conv, int row, int sec18, float m0, float m1) {
+                                            bool first, bool conv, float X, int sec18, float m0, float m1) {
   float chi2 = 0.0f;
   if (first) {
-    S.x = T.row_x[row];
+    S.x = X;
     S.sec = sec18;
     if (conv) {
       S.p[0] = S.p[0] - m0;
@@ -342,7 +342,7 @@ __device__ __forceinline__ void step_fwd_ud(const GeoRef& G, const SmemTables& T
     float pn[5];
     Jac J;
     PredTape tp;
-    if (predict_residual<FIELD>(G, T, S.p, S.x, S.sec, my, mz, sec18, T.row_x[row], m0, m1, pn, J, tp)) {
+    if (predict_residual<FIELD>(G, T, S.p, S.x, S.sec, my, mz, sec18, X, m0, m1, pn, J, tp)) {
 #pragma unroll
       for (int c = 0; c < 5; ++c) S.p[c] = pn[c];
       if (J.rot)
@@ -350,7 +350,7 @@ __device__ __forceinline__ void step_fwd_ud(const GeoRef& G, const SmemTables& T
       else
         transport_ud(S.u, J);
     }
-    S.x = T.row_x[row];
+    S.x = X;
     S.sec = sec18;
   }
   my = m0;
@@ -360,14 +360,15 @@ __device__ __forceinline__ void step_fwd_ud(const GeoRef& G, const SmemTables& T
 }
 
 // Reverse of one step in U-D form; the arguments as for step_rev, with the
-// factor's adjoint (b_u, b_d) in place of b_L, and x_prev, sec_prev (the
-// previous cluster's row position and sector mod 18: the state's frame).
+// factor's adjoint (b_u, b_d) in place of b_L, the row's x in place of its
+// number, and x_prev, sec_prev (the previous cluster's row position and sector
+// mod 18: the state's frame).
 // The gradient of the current cluster's measurement is handed to acc(g0, g1)
 // as soon as the update reverses have produced it, so that it is not held
 // through the reverses of the transport and the prediction.
 template <int FIELD = 0, class Acc>
 __device__ __forceinline__ void step_rev_ud(const GeoRef& G, const SmemTables& T, const float4* src, float my_prev,
-                                            float mz_prev, float x_prev, int sec_prev, bool first, bool conv, int row,
+                                            float mz_prev, float x_prev, int sec_prev, bool first, bool conv, float X,
                                             int sec18, float m0, float m1, float b_p[5], float b_u[10], float b_d[5],
                                             float b_chi, Acc&& acc, float b_mp[2]) {
   UDState S0;
@@ -387,7 +388,7 @@ __device__ __forceinline__ void step_rev_ud(const GeoRef& G, const SmemTables& T
       p1[1] = S0.p[1] - m1;
     }
   } else {
-    moved = predict_residual<FIELD>(G, T, S0.p, S0.x, S0.sec, my_prev, mz_prev, sec18, T.row_x[row], m0, m1, p1, J, tp);
+    moved = predict_residual<FIELD>(G, T, S0.p, S0.x, S0.sec, my_prev, mz_prev, sec18, X, m0, m1, p1, J, tp);
     if (!moved) {
 #pragma unroll
       for (int c = 0; c < 5; ++c) p1[c] = S0.p[c];
