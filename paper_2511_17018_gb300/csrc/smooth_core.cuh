@@ -13,7 +13,12 @@
 // form (smooth_combine).  Outputs: the residual m_c - H x_u,
 // R = V + H C_u H^T and chi2 = r^T R^-1 r (2 degrees of freedom).
 //
-// Work mapping: the outward filter runs forward from the seed, cluster by
+// Both predictions follow from states that the recorded fit left on its tape, so
+// the clusters of a track are smoothed independently of each other
+// (smooth_tape_kernel).  Items without a place on the tape go through
+// smooth_kernel, from the checkpoints:
+//
+// Work mapping of smooth_kernel: the outward filter runs forward from the seed, cluster by
 // cluster.  The inward predictions are needed in the same order, which is the
 // reverse of the inward pass; they come from the inward checkpoints segment by
 // segment (last segment first): a segment is recomputed into the warp's
@@ -227,66 +232,6 @@ __device__ __forceinline__ void write_nan_clusters(const SmoothArgs& a, int h0, 
   }
 }
 
-// The state before step i of a pass as the recorded fit left it: from the tape or
-// from its checkpoint (i a multiple of kCkptEvery).  Copied asynchronously into
-// the warp's lane-interleaved checkpoint buffer, as one commit group; a U-D
-// state's x and sector are those of the cluster before the step.
-struct RecordedPass {
-  const float4* src;       // tape: this lane's float4 of the pass's first state; checkpoints: the first one
-  const float4* cluster;   // U-D tape: this lane's cluster of step 0
-  int pitch;               // tape: tracks of the item; 0: checkpoints
-  int cluster_step;
-};
-
-__device__ __forceinline__ RecordedPass recorded_pass(const SmoothArgs& a, int2 place, int pass, int lane, int begin,
-                                                      int trk, int steps) {
-  RecordedPass r;
-  r.cluster = nullptr;
-  r.cluster_step = 0;
-  if (a.tape_item && place.x >= 0) {
-    r.pitch = a.item_tracks;
-    const float4* row0 = tape_row0(a.tape, place, r.pitch, lane);
-    if (a.ck_form == 1) {
-      r.src = row0 + (place.y + kUDRows * pass * (int)tape_states(place.y, a.tape_every)) * r.pitch;
-      r.cluster = row0 + (pass == 0 ? 0 : steps - 1) * r.pitch;
-      r.cluster_step = pass == 0 ? r.pitch : -r.pitch;
-    } else {
-      r.src = row0 + kSqrtRows * pass * place.y * r.pitch;
-    }
-  } else {
-    r.pitch = 0;
-    r.src = reinterpret_cast<const float4*>(a.ck + ((int64_t)pass * a.ck_slots + (begin >> kCkptShift) + trk) * kCkptFloats);
-  }
-  return r;
-}
-
-__device__ __forceinline__ void fetch_recorded(float4* sdst, const SmoothArgs& a, const RecordedPass& r, int i) {
-  if (r.pitch == 0) {
-    fetch_ckpt(sdst, reinterpret_cast<const float*>(r.src) + (int64_t)(i >> kCkptShift) * kCkptFloats);
-    return;
-  }
-  if (a.ck_form == 1) {
-    copy_rows<kUDRows>(sdst, r.src + i / a.tape_every * (kUDRows * r.pitch), r.pitch);
-    if (i > 0) cp_async16(sdst + kUDRows * kWarp, r.cluster + (i - 1) * r.cluster_step);
-  } else {
-    copy_rows<kSqrtRows>(sdst, r.src + i * (kSqrtRows * r.pitch), r.pitch);
-  }
-  cp_async_commit();
-}
-
-// The fetched state (after a wait), as the square-root factor.
-__device__ __forceinline__ void read_recorded(const float4* src, const SmoothArgs& a, const RecordedPass& r, int i,
-                                              StepState& S) {
-  read_state(src, S);
-  if (a.ck_form != 1) return;
-  sqrt_from_ud_ckpt(S);
-  if (r.pitch != 0 && i > 0) {
-    const float4 c = src[kUDRows * kWarp];
-    S.x = c.z;
-    S.sec = side_sector(__float_as_int(c.w) & 63);
-  }
-}
-
 // Shared memory of a smoother block: the tables, the alignment table and,
 // per warp, a double buffer for the inward states and a checkpoint buffer.
 template <int WARPS>
@@ -296,9 +241,37 @@ constexpr size_t smooth_smem_bytes() {
 
 // STATES: the smoothed state and its covariance at every cluster as well
 // (a.state, a.state_cov); without it the kernel carries none of that code.
+//
+// After a fit that left a U-D tape it does two things.  Items without a place on
+// the tape go through it whole.  Of the others it smooths the states of the last
+// kSmoothEnds clusters of each track, whose covariance depends on rounding at 3e-5
+// in norm (the inward prior is diffuse there: a cluster or two against 100 cm^2
+// and steep tracks): they keep the square-root sequence, along the outward filter
+// from the seed, and smooth_tape_kernel does the rest (30,000 tracks: 169 us for
+// the ends, 185 for the rest).
+constexpr int kSmoothEnds = kCkptEvery;
+
+// An outward or inward pass's first state from the U-D tape, as a checkpoint.
+__device__ __forceinline__ void tape_first_state(const float4* src, int pitch, StepState& S) {
+  float v[32];
+#pragma unroll
+  for (int e = 20; e < 32; ++e) v[e] = 0.0f;
+#pragma unroll
+  for (int j = 0; j < kUDRows; ++j) {
+    const float4 f = __ldg(src + j * pitch);
+    v[4 * j] = f.x;
+    v[4 * j + 1] = f.y;
+    v[4 * j + 2] = f.z;
+    v[4 * j + 3] = f.w;
+  }
+  unpack_state(v, S);
+}
+
 template <int WARPS, bool MAT, bool STATES>
 __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_constant__ SmoothArgs a) {
   const GeoRef& G = a.geo;
+  const bool ends_too = STATES && a.ck_form == 1;
+  if (a.tape_item && !ends_too && a.work[kWorkMissing] == 0) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdSmem& B = *reinterpret_cast<BwdSmem*>(smem_raw);
   load_block_tables(G, B.T, B.align, a.align);
@@ -312,98 +285,122 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
   for (bool first = true;; first = false) {
     const int64_t item = next_item(a.work, n_items, first);
     if (item < 0) break;
-    const int64_t slot = item * a.item_tracks + lane;
-    if (lane >= a.item_tracks || slot >= a.n_tracks) continue;
-    const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
-    const int begin = a.off[trk];
-    const int end = a.off[trk + 1];
-    if (a.ndf[trk] <= 0) {
-      write_nan_clusters(a, begin, end);
-      continue;
-    }
-    const int last = a.ck_last[trk];
-    write_nan_clusters(a, begin + last + 1, end);  // clusters the outward pass did not reach
     const int2 place = a.tape_item ? a.tape_item[item] : make_int2(-1, 0);
+    const bool ends = ends_too && place.x >= 0;
+    if (place.x >= 0 && !ends) continue;  // smooth_tape_kernel's
+    const int64_t slot = item * a.item_tracks + lane;
+    const bool have = lane < a.item_tracks && slot < a.n_tracks;
+    const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
+    const int begin = have ? a.off[trk] : 0;
+    const bool fitted = have && a.ndf[trk] > 0;
+    const int steps = fitted ? a.ck_last[trk] + 1 : 0;
+    const int last = steps - 1;
+    if (have && !ends) write_nan_clusters(a, begin + steps, a.off[trk + 1]);  // without an estimate
+    const int64_t slot0 = (begin >> kCkptShift) + trk;
+    const float4* const row0 = ends ? tape_row0(a.tape, place, a.item_tracks, lane) + place.y * a.item_tracks : nullptr;
     // outward filter: from its first state (the seed, factor L0)
     StepState O;
-    {
-      const RecordedPass out = recorded_pass(a, place, 0, lane, begin, trk, last + 1);
-      fetch_recorded(&W.ck[0][lane], a, out, 0);
-      cp_async_wait<0>();
-      read_recorded(&W.ck[0][lane], a, out, 0, O);
-    }
     float omy = 0.0f, omz = 0.0f;  // measurement O's residuals refer to (none for the seed)
     // inward segments, last first: inward step j is cluster last - j
-    const int steps = last + 1;
     const int nseg = (steps + kCkptEvery - 1) / kCkptEvery;
-    const RecordedPass in = recorded_pass(a, place, 1, lane, begin, trk, last + 1);
+    const float* ckp = a.ck + ((int64_t)a.ck_slots + slot0) * kCkptFloats;
     const int h_last = begin + last;
-    fetch_recorded(&W.ck[0][lane], a, in, (nseg - 1) * kCkptEvery);
+    HitRaw ahead{};  // the cluster after the one taken next
+    float m0 = 0.0f, m1 = 0.0f;
+    int row = 0, sec = 0;
+    if (fitted) {
+      if (ends) {
+        tape_first_state(row0, a.item_tracks, O);
+      } else {
+        fetch_ckpt(&W.ck[0][lane], a.ck + slot0 * kCkptFloats);
+        cp_async_wait<0>();
+        read_state(&W.ck[0][lane], O);
+        fetch_ckpt(&W.ck[0][lane], ckp + (int64_t)(nseg - 1) * kCkptFloats);
+      }
+      if (a.ck_form == 1) sqrt_from_ud_ckpt(O);
+      decode_hit(B.align, load_hit(a.y, a.z, a.rowsec, begin), m0, m1, row, sec);
+      if (last > 0) ahead = load_hit(a.y, a.z, a.rowsec, begin + 1);
+    }
+    // the segments of all lanes together, so that lanes of different lengths stay
+    // converged
 #pragma unroll 1
-    for (int s = nseg - 1; s >= 0; --s) {
+    for (int s = __reduce_max_sync(0xffffffffu, nseg) - 1; s >= 0; --s) {
+      __syncwarp();
+      if (s >= nseg) continue;
       const int j0 = s * kCkptEvery;
       const int cnt = min(kCkptEvery, steps - j0);
-      StepState S;
-      float my = 0.0f, mz = 0.0f;
-      HitRaw nx = load_hit(a.y, a.z, a.rowsec, h_last - j0);
-      if (j0 > 0) {
-        int row, sec;
-        decode_hit(B.align, load_hit(a.y, a.z, a.rowsec, h_last - (j0 - 1)), my, mz, row, sec);
-      }
-      cp_async_wait<0>();
-      read_recorded(&W.ck[0][lane], a, in, j0, S);
-      // level 1: the inward segment, storing the state before each step
+      const bool combine = !ends || s == 0;
+      if (combine) {
+        StepState S;
+        float my = 0.0f, mz = 0.0f;
+        HitRaw nx = load_hit(a.y, a.z, a.rowsec, h_last - j0);
+        if (j0 > 0) {
+          int prow, psec;
+          decode_hit(B.align, load_hit(a.y, a.z, a.rowsec, h_last - (j0 - 1)), my, mz, prow, psec);
+        }
+        if (ends) {
+          tape_first_state(row0 + kUDRows * (int)tape_states(place.y, a.tape_every) * a.item_tracks, a.item_tracks, S);
+        } else {
+          cp_async_wait<0>();
+          read_state(&W.ck[0][lane], S);
+        }
+        if (a.ck_form == 1) sqrt_from_ud_ckpt(S);
+        // level 1: the inward segment, storing the state before each step
 #pragma unroll 1
-      for (int kk = 0; kk < cnt; ++kk) {
-        const int j = j0 + kk;
-        const HitRaw cur = nx;
-        if (kk + 1 < cnt) nx = load_hit(a.y, a.z, a.rowsec, h_last - (j + 1));
-        float m0, m1;
-        int row, sec;
-        decode_hit(B.align, cur, m0, m1, row, sec);
-        store_state(gs + kk * (kStateF4 * kWarp), S);
-        step_fwd<MAT, 2>(G, T, S, my, mz, j == 0, false, row, side_sector(sec), m0, m1);
+        for (int kk = 0; kk < cnt; ++kk) {
+          const int j = j0 + kk;
+          const HitRaw cur = nx;
+          if (kk + 1 < cnt) nx = load_hit(a.y, a.z, a.rowsec, h_last - (j + 1));
+          float n0, n1;
+          int nrow, nsec;
+          decode_hit(B.align, cur, n0, n1, nrow, nsec);
+          store_state(gs + kk * (kStateF4 * kWarp), S);
+          step_fwd<MAT, 2>(G, T, S, my, mz, j == 0, false, nrow, side_sector(nsec), n0, n1);
+        }
+        __threadfence_block();  // the states just stored are read back by this thread's copies below
+        if (s > 0) fetch_ckpt(&W.ck[0][lane], ckp + (int64_t)(s - 1) * kCkptFloats);
+        fetch_state(&W.st[(cnt - 1) & 1][0][lane], gs + (cnt - 1) * (kStateF4 * kWarp));
       }
-      __threadfence_block();  // the states just stored are read back by this thread's copies below
-      if (s > 0) fetch_recorded(&W.ck[0][lane], a, in, (s - 1) * kCkptEvery);
-      fetch_state(&W.st[(cnt - 1) & 1][0][lane], gs + (cnt - 1) * (kStateF4 * kWarp));
       // consume in reverse: cluster c = last - j ascending
 #pragma unroll 1
       for (int kk = cnt - 1; kk >= 0; --kk) {
         const int j = j0 + kk;
         const int c = last - j;
         const int h = begin + c;
-        if (kk > 0) {
-          fetch_state(&W.st[(kk - 1) & 1][0][lane], gs + (kk - 1) * (kStateF4 * kWarp));
-          cp_async_wait<1>();
-        } else {
-          cp_async_wait<0>();
-        }
-        float m0, m1;
-        int row, sec;
-        decode_hit(B.align, load_hit(a.y, a.z, a.rowsec, h), m0, m1, row, sec);
         const int sec18 = side_sector(sec);
         const float X = T.row_x[row];
+        // the cluster after this one
+        float mpy = 0.0f, mpz = 0.0f;
+        int prow = 0, psec = 0;
+        if (j > 0) {
+          decode_hit(B.align, ahead, mpy, mpz, prow, psec);
+          if (j > 1) ahead = load_hit(a.y, a.z, a.rowsec, h + 2);
+        }
         // inward prediction at c
         StepState SI;
-        read_state(&W.st[kk & 1][0][lane], SI);
         float pi[5];
-        if (j == 0) {  // the inward pass starts on this cluster
-#pragma unroll
-          for (int q = 0; q < 5; ++q) pi[q] = SI.p[q];
-        } else {
-          float mpy, mpz;
-          int prow, psec;
-          decode_hit(B.align, load_hit(a.y, a.z, a.rowsec, h + 1), mpy, mpz, prow, psec);
-          Jac J;
-          PredTape tp;
-          if (MAT) {  // the layer of row c + 1, undone against the flight
-            MatNoise N;
-            material_step(G, SI.p, -1, N);
-            material_factor(SI.L, N);
+        if (combine) {
+          if (kk > 0) {
+            fetch_state(&W.st[(kk - 1) & 1][0][lane], gs + (kk - 1) * (kStateF4 * kWarp));
+            cp_async_wait<1>();
+          } else {
+            cp_async_wait<0>();
           }
-          predict_residual<2>(G, T, SI.p, SI.x, SI.sec, mpy, mpz, sec18, X, m0, m1, pi, J, tp);
-          transport(SI.L, J);
+          read_state(&W.st[kk & 1][0][lane], SI);
+          if (j == 0) {  // the inward pass starts on this cluster
+#pragma unroll
+            for (int q = 0; q < 5; ++q) pi[q] = SI.p[q];
+          } else {
+            Jac J;
+            PredTape tp;
+            if (MAT) {  // the layer of row c + 1, undone against the flight
+              MatNoise N;
+              material_step(G, SI.p, -1, N);
+              material_factor(SI.L, N);
+            }
+            predict_residual<2>(G, T, SI.p, SI.x, SI.sec, mpy, mpz, sec18, X, m0, m1, pi, J, tp);
+            transport(SI.L, J);
+          }
         }
         // outward prediction at c
         float po[5];
@@ -440,7 +437,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
         float chi_unused = 0.0f;
         scalar_update<0>(G, O.p, O.L, chi_unused, 0.0f);
         scalar_update<1>(G, O.p, O.L, chi_unused, 0.0f);
-        if (STATES) {  // the outward filtered state at c with the inward prediction
+        if (STATES && combine) {  // the outward filtered state at c with the inward prediction
           float xs[5], Cs[15];
           smooth_state(O.p, O.L, pi, SI.L, xs, Cs);
           xs[0] = xs[0] + m0;  // residual coordinates back to positions
@@ -450,7 +447,400 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
 #pragma unroll
           for (int q = 0; q < 15; ++q) a.state_cov[(int64_t)h * 15 + q] = Cs[q];
         }
+        m0 = mpy;
+        m1 = mpz;
+        row = prow;
+        sec = psec;
       }
+    }
+  }
+}
+
+// ---------------------------------------------------------------- from the tape
+// The two estimates of a state in U-D form combined: the second one, (p2, U2, D2),
+// is five measurements V p2 of the state with V = U2^-1 (unit upper triangular)
+// and independent errors of variance D2, taken by the first one, (p, U, D), in
+// turn with Bierman's scalar update (bierman_update with row k of V in place of a
+// unit vector).  About 330 operations; no sum of the covariances is formed, and
+// next to a diffuse end of the track, where one side is a cluster or two and the
+// prior, the variances stay in D, apart from each other: the covariances are
+// closer to 64 bits than those of the orthogonal reduction.
+template <int K>
+__device__ __forceinline__ void take_component(float p[5], float u[10], float d[5], const float p2[5], const float V[10],
+                                               float variance) {
+  float gain[5];
+  float ap = variance, iap = 0.0f;
+  float r = p2[K] - p[K];
+#pragma unroll
+  for (int i = K + 1; i < 5; ++i) r = r + V[ui(K, i)] * (p2[i] - p[i]);
+#pragma unroll
+  for (int j = K; j < 5; ++j) {
+    float f = 1.0f;  // column j of U against row K of V
+    if (j > K) {
+      f = V[ui(K, j)] + u[ui(K, j)];
+#pragma unroll
+      for (int i = K + 1; i < j; ++i) f = f + V[ui(K, i)] * u[ui(i, j)];
+    }
+    const float g = j == K ? d[j] : d[j] * f;
+    const float a = j == K ? ap + g : ap + f * g;
+    const float ia = ud_rcp(a);
+    if (j > K) {
+      const float lam = -(f * iap);
+#pragma unroll
+      for (int i = 0; i < j; ++i) {
+        const float uo = u[ui(i, j)];
+        u[ui(i, j)] = uo + lam * gain[i];
+        gain[i] = gain[i] + g * uo;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < j; ++i) gain[i] = g * u[ui(i, j)];
+    }
+    d[j] = d[j] * (ap * ia);
+    gain[j] = g;
+    ap = a;
+    iap = ia;
+  }
+  const float q = r * iap;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) p[i] = p[i] + gain[i] * q;
+}
+
+__device__ __forceinline__ void combine_ud(float p[5], float u[10], float d[5], const float p2[5], const float u2[10],
+                                           const float d2[5]) {
+  float V[10];  // U2^-1
+#pragma unroll
+  for (int i = 3; i >= 0; --i)
+#pragma unroll
+    for (int j = i + 1; j < 5; ++j) {
+      float acc = u2[ui(i, j)];
+#pragma unroll
+      for (int k = i + 1; k < j; ++k) acc = acc + u2[ui(i, k)] * V[ui(k, j)];
+      V[ui(i, j)] = -acc;
+    }
+  take_component<4>(p, u, d, p2, V, d2[4]);
+  take_component<3>(p, u, d, p2, V, d2[3]);
+  take_component<2>(p, u, d, p2, V, d2[2]);
+  take_component<1>(p, u, d, p2, V, d2[1]);
+  take_component<0>(p, u, d, p2, V, d2[0]);
+}
+
+// Every cluster on its own: the state before the outward step to it and the one
+// before the inward step to it come from the tape (with every second state there,
+// an odd one is recomputed from the one before it), are predicted to the cluster
+// and combined.  A unit of work is a few consecutive clusters of an item's
+// tracks, one track per lane.  No lane waits for another cluster, where
+// smooth_kernel recomputes both filters along each track.
+//
+// Bound by its arithmetic and by instruction fetch: the two predictions of a
+// cluster are two turns of one loop, since two copies of the prediction and the
+// recomputed step miss the instruction cache (1.4 warps waiting for instructions
+// per issue, 0.3 as a loop).  Measured: leave-one-out residuals of 100,000 tracks
+// 823 -> 465 us, smoothed states of 30,000 tracks, the ends included, 675 -> 358 us.
+// The unit's clusters are copied into shared memory once and each state one turn
+// ahead; the outputs leave through shared memory too, a track's run of clusters at
+// a time instead of single words.
+template <bool STATES>
+struct SmoothOut {
+  static constexpr int kSteps = STATES ? 4 : 8;         // clusters of a track in a unit
+  static constexpr int kUnits = kMaxRows / kSteps;      // units of an item (longer tracks: again)
+  static constexpr int kFloats = STATES ? 20 : 6;       // per cluster: (state 5, cov 15) or (resid 2, rcov 3, chi2)
+  static constexpr int kPitch = kFloats * kSteps + 1;   // odd: lanes fall into different banks
+  float v[kWarp][kPitch];
+  int first[kWarp];  // the unit's first cluster of each track, and how many
+  int count[kWarp];
+};
+
+// Per warp: the outputs and, in U-D form, the unit's clusters with two more on
+// either side and two states (one in use, one on its way).
+template <bool STATES, int FORM>
+struct SmoothWarp {
+  SmoothOut<STATES> out;
+};
+template <bool STATES>
+struct SmoothWarp<STATES, 1> {
+  static constexpr int kClusters = SmoothOut<STATES>::kSteps + 4;
+  alignas(16) float4 cluster[kClusters][kWarp];
+  float4 state[2][kUDRows][kWarp];
+  SmoothOut<STATES> out;
+};
+
+// One output of the unit: PER floats to a cluster, at AT in the cluster's record.
+// 32 consecutive lanes write consecutive words of a track's run.
+template <class Out, int PER, int AT>
+__device__ __forceinline__ void write_unit(float* dst, const Out& O, int tracks, int lane) {
+  constexpr int kRun = Out::kSteps * PER;
+  int t = lane / kRun, r = lane % kRun;  // track and word of its run
+#pragma unroll 4
+  for (int e = lane; e < tracks * kRun; e += kWarp) {
+    const int c = r / PER;
+    if (c < O.count[t]) dst[(int64_t)O.first[t] * PER + r] = O.v[t][c * Out::kFloats + AT + (r - c * PER)];
+    t += kWarp / kRun;
+    r += kWarp % kRun;
+    if (r >= kRun) {
+      r -= kRun;
+      ++t;
+    }
+  }
+}
+
+template <int WARPS, int FORM, bool MAT, bool STATES>
+__global__ void __launch_bounds__(WARPS * 32, 1) smooth_tape_kernel(const __grid_constant__ SmoothArgs a) {
+  const GeoRef& G = a.geo;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  // the square-root tape holds no clusters: they need the alignment table
+  constexpr size_t kBlock = FORM == 1 ? sizeof(SmemTables) : sizeof(BwdSmem);
+  BwdSmem& B = *reinterpret_cast<BwdSmem*>(smem_raw);
+  load_block_tables(G, B.T, B.align, FORM == 1 ? nullptr : a.align);
+  const SmemTables& T = B.T;
+  const int lane = threadIdx.x & 31;
+  using Out = SmoothOut<STATES>;
+  using Warp = SmoothWarp<STATES, FORM>;
+  Warp& W = reinterpret_cast<Warp*>(smem_raw + kBlock)[threadIdx.x >> 5];
+  Out& O = W.out;
+  const int pitch = a.item_tracks;
+  const int64_t n_items = ((int64_t)a.n_tracks + pitch - 1) / pitch;
+#pragma unroll 1
+  for (bool first = true;; first = false) {
+    const int64_t unit = next_item(a.work, n_items * Out::kUnits, first);
+    if (unit < 0) break;
+    const int64_t item = unit / Out::kUnits;
+    const int part = (int)(unit % Out::kUnits);
+    const int2 place = a.tape_item[item];
+    if (place.x < 0) continue;  // smooth_kernel's
+    const int64_t slot = item * pitch + lane;
+    const bool have = lane < pitch && slot < a.n_tracks;
+    const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
+    const int begin = have ? a.off[trk] : 0;
+    const bool fitted = have && a.ndf[trk] > 0;
+    const int steps = fitted ? a.ck_last[trk] + 1 : 0;
+    if (have && part == 0) write_nan_clusters(a, begin + steps, a.off[trk + 1]);  // without an estimate
+    // the states of a track's last clusters are smooth_kernel's (U-D form)
+    const int upto = STATES && FORM == 1 ? max(0, steps - kSmoothEnds) : steps;
+    const int most = __reduce_max_sync(0xffffffffu, upto);
+    const float4* const row0 = tape_row0(a.tape, place, pitch, lane);
+    const int every = FORM == 1 ? a.tape_every : 1;
+    const int states = (int)tape_states(place.y, every);
+
+    // a track's cluster: measured (y, z), the row's x, sector mod 18
+    struct At {
+      float m0, m1, X;
+      int sec;
+    };
+#pragma unroll 1
+    for (int c0 = part * Out::kSteps; c0 < most; c0 += Out::kUnits * Out::kSteps) {
+      if constexpr (FORM == 1) {
+#pragma unroll 1
+        for (int e = 0; e < Warp::kClusters; ++e) {
+          const int c = c0 - 2 + e;
+          if (c >= 0 && c < steps) cp_async16(&W.cluster[e][lane], row0 + c * pitch);
+        }
+        auto cluster = [&](int c) {
+          const float4 v = W.cluster[c - c0 + 2][lane];
+          At k;
+          k.m0 = v.x;
+          k.m1 = v.y;
+          k.X = v.z;
+          k.sec = side_sector(__float_as_int(v.w) & 63);
+          return k;
+        };
+        // turn q: cluster c0 + q / 2, the inward prediction first
+        auto fetch = [&](int q) {
+          const int c = c0 + (q >> 1), pass = 1 - (q & 1);
+          if (q < 2 * Out::kSteps && c < upto) {
+            const int i = pass == 0 ? c : steps - 1 - c;
+            copy_rows<kUDRows>(&W.state[q & 1][0][lane],
+                               row0 + (place.y + kUDRows * (pass * states + (every == 2 ? i >> 1 : i))) * pitch, pitch);
+          }
+          cp_async_commit();
+        };
+        fetch(0);
+        float p2[5], u2[10], d2[5];
+#pragma unroll 1
+        for (int q = 0; q < 2 * Out::kSteps; ++q) {
+          fetch(q + 1);
+          cp_async_wait<1>();
+          const int c = c0 + (q >> 1), pass = 1 - (q & 1);
+          if (c >= upto) continue;
+          const At at = cluster(c);
+          const int dir = pass == 0 ? 1 : -1;  // from one step's cluster to the next
+          const int i = pass == 0 ? c : steps - 1 - c;
+          UDState S;
+          read_state_ud<false>(&W.state[q & 1][0][lane], S);
+          At prev = at;  // the state's own cluster
+          if (i > 0) prev = cluster(c - dir);
+          if (every == 2 && (i & 1)) {  // from the state before: its step, to cluster prev
+            At pp = prev;
+            if (i > 1) pp = cluster(c - 2 * dir);
+            S.x = pp.X;
+            S.sec = pp.sec;
+            float my = pp.m0, mz = pp.m1;
+            step_fwd_ud<2>(G, T, S, my, mz, i == 1, pass == 0, prev.X, prev.sec, prev.m0, prev.m1);
+          }
+          S.x = prev.X;
+          S.sec = prev.sec;
+          float pn[5];
+          if (i == 0) {  // the pass starts on this cluster (outward: the seed, absolute)
+#pragma unroll
+            for (int e = 0; e < 5; ++e) pn[e] = S.p[e];
+            if (pass == 0) {
+              pn[0] = S.p[0] - at.m0;
+              pn[1] = S.p[1] - at.m1;
+            }
+          } else {
+            Jac J;
+            PredTape tp;
+            predict_residual<2>(G, T, S.p, S.x, S.sec, prev.m0, prev.m1, at.sec, at.X, at.m0, at.m1, pn, J, tp);
+            if (J.rot)
+              rotate_ud(S.u, S.d, J);
+            else
+              transport_ud(S.u, J);
+          }
+          if (pass == 1) {
+#pragma unroll
+            for (int e = 0; e < 5; ++e) p2[e] = pn[e];
+#pragma unroll
+            for (int e = 0; e < 10; ++e) u2[e] = S.u[e];
+#pragma unroll
+            for (int e = 0; e < 5; ++e) d2[e] = S.d[e];
+            continue;
+          }
+          if (STATES) {  // the outward filtered state: with cluster c
+            float chi_unused = 0.0f;
+            bierman_update<0>(pn, S.u, S.d, chi_unused, G.v_meas);
+            bierman_update<1>(pn, S.u, S.d, chi_unused, G.v_meas);
+          }
+          combine_ud(pn, S.u, S.d, p2, u2, d2);
+          float* const o = &O.v[lane][(q >> 1) * Out::kFloats];
+          if (STATES) {
+            o[0] = pn[0] + at.m0;  // residual coordinates back to positions
+            o[1] = pn[1] + at.m1;
+#pragma unroll
+            for (int e = 2; e < 5; ++e) o[e] = pn[e];
+            int n = 5;
+#pragma unroll
+            for (int r = 0; r < 5; ++r)
+#pragma unroll
+              for (int j = 0; j <= r; ++j) {
+                float acc = (j == r ? 1.0f : S.u[ui(j, r)]) * S.d[r];
+#pragma unroll
+                for (int k = r + 1; k < 5; ++k) acc = acc + (S.u[ui(r, k)] * S.d[k]) * S.u[ui(j, k)];
+                o[n++] = acc;
+              }
+          } else {
+            // the state is relative to the measurement: r = m - H x_u = -(y, z)
+            const float r0 = -pn[0], r1 = -pn[1];
+            float R0 = S.d[0], R1 = S.u[ui(0, 1)] * S.d[1], R2 = S.d[1];
+#pragma unroll
+            for (int k = 1; k < 5; ++k) R0 = R0 + (S.u[ui(0, k)] * S.d[k]) * S.u[ui(0, k)];
+#pragma unroll
+            for (int k = 2; k < 5; ++k) {
+              R1 = R1 + (S.u[ui(1, k)] * S.d[k]) * S.u[ui(0, k)];
+              R2 = R2 + (S.u[ui(1, k)] * S.d[k]) * S.u[ui(1, k)];
+            }
+            R0 = R0 + G.v_meas;
+            R2 = R2 + G.v_meas;
+            const float det = R0 * R2 - R1 * R1;
+            o[0] = r0;
+            o[1] = r1;
+            o[2] = R0;
+            o[3] = R1;
+            o[4] = R2;
+            o[5] = (R2 * r0 * r0 - 2.0f * R1 * r0 * r1 + R0 * r1 * r1) / det;
+          }
+        }
+        cp_async_wait<0>();
+      } else {
+        auto cluster = [&](int c) {
+          At k;
+          int row, sec;
+          decode_hit(B.align, load_hit(a.y, a.z, a.rowsec, begin + c), k.m0, k.m1, row, sec);
+          k.X = T.row_x[row];
+          k.sec = side_sector(sec);
+          return k;
+        };
+#pragma unroll 1
+        for (int k = 0; k < Out::kSteps; ++k) {
+          const int c = c0 + k;
+          if (c >= upto) continue;
+          const At at = cluster(c);
+          float* const o = &O.v[lane][k * Out::kFloats];
+          float pp[2][5];
+          StepState S[2];
+#pragma unroll
+          for (int pass = 1; pass >= 0; --pass) {
+            const int i = pass == 0 ? c : steps - 1 - c;
+            const float4* src = row0 + kSqrtRows * (pass * place.y + i) * pitch;
+            {
+              float v[32];
+#pragma unroll
+              for (int j = 0; j < kSqrtRows; ++j) {
+                const float4 f = __ldg(src + j * pitch);
+                v[4 * j] = f.x;
+                v[4 * j + 1] = f.y;
+                v[4 * j + 2] = f.z;
+                v[4 * j + 3] = f.w;
+              }
+              unpack_state(v, S[pass]);
+            }
+            if (i == 0) {
+#pragma unroll
+              for (int q = 0; q < 5; ++q) pp[pass][q] = S[pass].p[q];
+              if (pass == 0) {
+                pp[0][0] = S[0].p[0] - at.m0;
+                pp[0][1] = S[0].p[1] - at.m1;
+              }
+            } else {
+              const At prev = cluster(pass == 0 ? c - 1 : c + 1);
+              Jac J;
+              PredTape tp;
+              MatNoise N;
+              if (MAT && pass == 1) {  // the layer of row c + 1, undone against the flight
+                material_step(G, S[1].p, -1, N);
+                material_factor(S[1].L, N);
+              }
+              predict_residual<2>(G, T, S[pass].p, S[pass].x, S[pass].sec, prev.m0, prev.m1, at.sec, at.X, at.m0,
+                                  at.m1, pp[pass], J, tp);
+              if (MAT && pass == 0) material_step(G, pp[0], 1, N);  // the layer of row c
+              transport(S[pass].L, J);
+              if (MAT && pass == 0) material_factor(S[0].L, N);
+            }
+          }
+          if (STATES) {
+            float chi_unused = 0.0f;
+            scalar_update<0>(G, pp[0], S[0].L, chi_unused, 0.0f);
+            scalar_update<1>(G, pp[0], S[0].L, chi_unused, 0.0f);
+            float xs[5], Cs[15];
+            smooth_state(pp[0], S[0].L, pp[1], S[1].L, xs, Cs);
+            o[0] = xs[0] + at.m0;
+            o[1] = xs[1] + at.m1;
+#pragma unroll
+            for (int q = 2; q < 5; ++q) o[q] = xs[q];
+#pragma unroll
+            for (int q = 0; q < 15; ++q) o[5 + q] = Cs[q];
+          } else {
+            float r[2], R[3], c2;
+            smooth_combine(G, pp[0], S[0].L, pp[1], S[1].L, r, R, c2);
+            o[0] = r[0];
+            o[1] = r[1];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) o[2 + q] = R[q];
+            o[5] = c2;
+          }
+        }
+      }
+      O.first[lane] = begin + c0;
+      O.count[lane] = max(0, min(Out::kSteps, upto - c0));
+      __syncwarp();
+      if (STATES) {
+        write_unit<Out, 5, 0>(a.state, O, pitch, lane);
+        write_unit<Out, 15, 5>(a.state_cov, O, pitch, lane);
+      } else {
+        write_unit<Out, 2, 0>(a.resid, O, pitch, lane);
+        write_unit<Out, 3, 2>(a.rcov, O, pitch, lane);
+        write_unit<Out, 1, 5>(a.chi2, O, pitch, lane);
+      }
+      __syncwarp();
     }
   }
 }
@@ -490,10 +880,49 @@ cudaError_t launch_smooth_cfg(const SmoothArgs& a, cudaStream_t s) {
                            sizeof(BwdSmem), sizeof(BwdWarpBufs), a, s);
 }
 
+constexpr int kSmoothTapeSqrtWarps = 8;
+
+template <int WARPS, int FORM, bool MAT, bool STATES>
+cudaError_t launch_smooth_tape(const SmoothArgs& a, cudaStream_t s) {
+  constexpr size_t kBlock = FORM == 1 ? sizeof(SmemTables) : sizeof(BwdSmem);
+  static Resident r;
+  auto kernel = smooth_tape_kernel<WARPS, FORM, MAT, STATES>;
+  cudaError_t e = resident_blocks(kernel, WARPS * kWarp, kBlock + WARPS * sizeof(SmoothWarp<STATES, FORM>), r);
+  if (e != cudaSuccess) return e;
+  SmoothArgs b = a;
+  b.item_tracks = item_tracks(a.n_tracks, r.sms);
+  const int64_t units = ((int64_t)a.n_tracks + b.item_tracks - 1) / b.item_tracks * SmoothOut<STATES>::kUnits;
+  const int blocks = (int)(units < r.blocks ? units : r.blocks);
+  const int64_t per_block = (units + blocks - 1) / blocks;
+  const int warps = (int)(per_block < WARPS ? per_block : WARPS);
+  e = clear_work(a.work, false, units > (int64_t)blocks * warps, s);
+  if (e != cudaSuccess) return e;
+  kernel<<<blocks, warps * kWarp, kBlock + warps * sizeof(SmoothWarp<STATES, FORM>), s>>>(b);
+  return cudaGetLastError();
+}
+
+template <bool STATES>
+cudaError_t launch_smooth_of(const SmoothArgs& a, cudaStream_t s) {
+  if (a.tape) {
+    cudaError_t e;
+#if !TPCFIT_DET
+    if (a.ck_form == 1)
+      e = launch_smooth_tape<STATES ? 10 : 12, 1, false, STATES>(a, s);
+    else  // the fast square-root form is on the tape with material layers only
+      e = launch_smooth_tape<kSmoothTapeSqrtWarps, 0, true, STATES>(a, s);
+#else
+    e = a.mat ? launch_smooth_tape<kSmoothTapeSqrtWarps, 0, true, STATES>(a, s)
+              : launch_smooth_tape<kSmoothTapeSqrtWarps, 0, false, STATES>(a, s);
+#endif
+    if (e != cudaSuccess) return e;
+  }
+  // from checkpoints: everything, or the items that the tape had no room for
+  return a.mat ? launch_smooth_cfg<true, STATES>(a, s) : launch_smooth_cfg<false, STATES>(a, s);
+}
+
 inline cudaError_t launch_smooth(const SmoothArgs& a, cudaStream_t s) {
   if (a.n_tracks <= 0) return cudaSuccess;
-  if (a.state) return a.mat ? launch_smooth_cfg<true, true>(a, s) : launch_smooth_cfg<false, true>(a, s);
-  return a.mat ? launch_smooth_cfg<true, false>(a, s) : launch_smooth_cfg<false, false>(a, s);
+  return a.state ? launch_smooth_of<true>(a, s) : launch_smooth_of<false>(a, s);
 }
 #endif
 
