@@ -140,9 +140,11 @@ int64_t reject_scratch_ints(int32_t n_tracks);
 cudaError_t launch_reject(const int32_t* off, int32_t n_tracks, const float* y, const float* z, const uint16_t* rowsec,
                           int64_t n_hits, const float* chi2, float cut, float* y_out, float* z_out,
                           uint16_t* rowsec_out, int32_t* off_out, int32_t* scratch, cudaStream_t s);
-// Exclusive prefix sum of n ints in place (key_reduce.cu); tmp: scan_tmp_ints(n) ints.
+// Exclusive prefix sum of n ints in place (key_reduce.cu); tmp: scan_tmp_ints(n)
+// ints, or null (one block does it whatever n; total, if not null, then receives
+// the sum of all).
 int64_t scan_tmp_ints(int64_t n);
-cudaError_t launch_scan_exclusive(int* v, int n, int* tmp, cudaStream_t s);
+cudaError_t launch_scan_exclusive(int* v, int n, int* total, int* tmp, cudaStream_t s);
 
 // Length-ordering permutation: perm[k] = track processed k-th, longest first.
 // scratch: int32[2 * 256] (zeroed by the launcher).

@@ -123,6 +123,54 @@ __global__ void __launch_bounds__(1024) scan_add(int* v, int n, const int* tile_
     if (base + i < n) v[base + i] += add;
 }
 
+// Exclusive prefix sum in place by one block, 4,096 ints at a time, and the sum of
+// all of them; in place of three kernels where that is fewer than 17 rounds.
+constexpr int kScanThreads = 1024;
+constexpr int kScanOneBlock = 65536;
+__global__ void __launch_bounds__(kScanThreads) scan_one_block(int* sums, int n, int* total) {
+  __shared__ int warp_tot[kScanThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int carry = 0;
+  for (int base = 0; base < n; base += 4 * kScanThreads) {
+    int v[4];
+    int mine = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = base + 4 * threadIdx.x + j;
+      v[j] = i < n ? sums[i] : 0;
+      mine += v[j];
+    }
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) warp_tot[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      int t = warp_tot[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, t, o);
+        if (lane >= o) t += u;
+      }
+      warp_tot[lane] = t;  // inclusive
+    }
+    __syncthreads();
+    int at = carry + (warp ? warp_tot[warp - 1] : 0) + incl - mine;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = base + 4 * threadIdx.x + j;
+      if (i < n) sums[i] = at;
+      at += v[j];
+    }
+    carry += warp_tot[kScanThreads / 32 - 1];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0 && total) *total = carry;
+}
+
 __global__ void __launch_bounds__(kThreads) radix_scatter(const uint16_t* rowsec, int n, int n_rows, const int* in,
                                                           int* out, int pass, const int* offsets, int nblocks) {
   __shared__ int run[kDigits];               // running count per digit within the block
@@ -228,8 +276,11 @@ cudaError_t launch_key_sort(const uint16_t* rowsec, int64_t n_hits, int n_rows, 
 
 int64_t scan_tmp_ints(int64_t n) { return (n + kScanTile - 1) / kScanTile + 1; }
 
-cudaError_t launch_scan_exclusive(int* v, int n, int* tmp, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
+cudaError_t launch_scan_exclusive(int* v, int n, int* total, int* tmp, cudaStream_t s) {
+  if (n <= kScanOneBlock || !tmp) {
+    scan_one_block<<<1, kScanThreads, 0, s>>>(v, n, total);
+    return cudaGetLastError();
+  }
   const int n_tiles = (n + kScanTile - 1) / kScanTile;
   scan_tiles<<<n_tiles, 1024, 0, s>>>(v, n, tmp);
   scan_totals<<<1, 1024, 0, s>>>(tmp, n_tiles);

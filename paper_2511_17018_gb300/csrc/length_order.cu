@@ -159,7 +159,7 @@ cudaError_t launch_frame_length_order(const int32_t* off, int32_t n_tracks, cons
   if (e != cudaSuccess) return e;
   const int64_t blocks = ((int64_t)n_tracks + 255) / 256;
   frame_hist<<<(unsigned)blocks, 256, 0, s>>>(off, n_tracks, frame_base, n_frames, start);
-  e = launch_scan_exclusive(start, (int)bins, tmp, s);
+  e = launch_scan_exclusive(start, (int)bins, nullptr, tmp, s);
   if (e != cudaSuccess) return e;
   frame_scatter<<<(unsigned)blocks, 256, 0, s>>>(off, n_tracks, frame_base, n_frames, start, cursor, perm);
   return cudaGetLastError();
