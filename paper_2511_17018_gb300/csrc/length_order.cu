@@ -121,24 +121,79 @@ __global__ void __launch_bounds__(kThreads) length_scatter(const int32_t* off, i
 }
 
 // Batched frames: key = frame * 256 + (255 - length) orders by frame, then by
-// decreasing length.  Histogram with global atomics, exclusive scan, scatter.
-__device__ __forceinline__ int frame_key(const int32_t* off, const int64_t* fb, int n_frames, int64_t i) {
-  int f = frame_of(fb, n_frames, i);
-  if (f < 0) f = n_frames - 1;  // out-of-table tracks are rejected by the fit; keep them in range here
-  return f * kBins + (kBins - 1 - length_bin(off, i));
+// decreasing length.  A block's tracks are consecutive, so nearly all of them are
+// in the frame of its first one (a second one at a boundary): those are counted in
+// shared memory and the block adds one count per length to the frame's, instead of
+// one global atomic per track on a few hundred addresses (40 frames, 576,000
+// tracks: histogram and scatter 18 + 23 us before).
+__device__ __forceinline__ int frame_clamped(const int64_t* fb, int n_frames, int64_t i) {
+  const int f = frame_of(fb, n_frames, i);
+  return f < 0 ? n_frames - 1 : f;  // out-of-table tracks are rejected by the fit; keep them in range here
 }
 
-__global__ void frame_hist(const int32_t* off, int32_t n, const int64_t* fb, int n_frames, int32_t* hist) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) atomicAdd(&hist[frame_key(off, fb, n_frames, i)], 1);
+// Frame of track i, given that of a track before it in the block.
+__device__ __forceinline__ int frame_near(const int64_t* fb, int n_frames, int64_t i, int f0, int64_t end0) {
+  return i < end0 ? f0 : frame_clamped(fb, n_frames, i);
 }
 
-__global__ void frame_scatter(const int32_t* off, int32_t n, const int64_t* fb, int n_frames, const int32_t* start,
-                              int32_t* cursor, int32_t* perm) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int k = frame_key(off, fb, n_frames, i);
-  perm[start[k] + atomicAdd(&cursor[k], 1)] = (int32_t)i;
+__global__ void __launch_bounds__(kThreads) frame_hist(const int32_t* off, int32_t n, const int64_t* fb, int n_frames,
+                                                       int32_t* hist) {
+  __shared__ int sh[kBins];
+  sh[threadIdx.x] = 0;
+  const int64_t first = (int64_t)blockIdx.x * kThreads * kItems;
+  const int f0 = frame_clamped(fb, n_frames, first);
+  const int64_t end0 = fb[f0 + 1];
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < kItems; ++it) {
+    const int64_t i = first + (int64_t)it * kThreads + threadIdx.x;
+    if (i >= n) continue;
+    const int f = frame_near(fb, n_frames, i, f0, end0);
+    const int bin = kBins - 1 - length_bin(off, i);
+    if (f == f0) atomicAdd(&sh[bin], 1);
+    else atomicAdd(&hist[f * kBins + bin], 1);
+  }
+  __syncthreads();
+  if (sh[threadIdx.x]) atomicAdd(&hist[f0 * kBins + threadIdx.x], sh[threadIdx.x]);
+}
+
+__global__ void __launch_bounds__(kThreads) frame_scatter(const int32_t* off, int32_t n, const int64_t* fb,
+                                                          int n_frames, const int32_t* start, int32_t* cursor,
+                                                          int32_t* perm) {
+  __shared__ int local[kBins];
+  __shared__ int base[kBins];
+  local[threadIdx.x] = 0;
+  const int64_t first = (int64_t)blockIdx.x * kThreads * kItems;
+  const int f0 = frame_clamped(fb, n_frames, first);
+  const int64_t end0 = fb[f0 + 1];
+  __syncthreads();
+  int bin[kItems], rank[kItems];
+#pragma unroll
+  for (int it = 0; it < kItems; ++it) {
+    const int64_t i = first + (int64_t)it * kThreads + threadIdx.x;
+    bin[it] = -1;
+    if (i >= n) continue;
+    const int f = frame_near(fb, n_frames, i, f0, end0);
+    const int k = kBins - 1 - length_bin(off, i);
+    if (f == f0) {
+      bin[it] = k;
+      rank[it] = atomicAdd(&local[k], 1);
+    } else {
+      const int key = f * kBins + k;
+      perm[start[key] + atomicAdd(&cursor[key], 1)] = (int32_t)i;
+    }
+  }
+  __syncthreads();
+  {
+    const int k = threadIdx.x;
+    base[k] = local[k] ? start[f0 * kBins + k] + atomicAdd(&cursor[f0 * kBins + k], local[k]) : 0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < kItems; ++it) {
+    const int64_t i = first + (int64_t)it * kThreads + threadIdx.x;
+    if (bin[it] >= 0) perm[base[bin[it]] + rank[it]] = (int32_t)i;
+  }
 }
 
 }  // namespace
@@ -157,11 +212,11 @@ cudaError_t launch_frame_length_order(const int32_t* off, int32_t n_tracks, cons
   int32_t* tmp = scratch + 2 * bins;
   cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int32_t) * 2 * bins, s);
   if (e != cudaSuccess) return e;
-  const int64_t blocks = ((int64_t)n_tracks + 255) / 256;
-  frame_hist<<<(unsigned)blocks, 256, 0, s>>>(off, n_tracks, frame_base, n_frames, start);
+  const int64_t blocks = ((int64_t)n_tracks + kThreads * kItems - 1) / (kThreads * kItems);
+  frame_hist<<<(unsigned)blocks, kThreads, 0, s>>>(off, n_tracks, frame_base, n_frames, start);
   e = launch_scan_exclusive(start, (int)bins, nullptr, tmp, s);
   if (e != cudaSuccess) return e;
-  frame_scatter<<<(unsigned)blocks, 256, 0, s>>>(off, n_tracks, frame_base, n_frames, start, cursor, perm);
+  frame_scatter<<<(unsigned)blocks, kThreads, 0, s>>>(off, n_tracks, frame_base, n_frames, start, cursor, perm);
   return cudaGetLastError();
 }
 
