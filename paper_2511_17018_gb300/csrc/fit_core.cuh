@@ -17,10 +17,10 @@
 // row with its Jacobian, L <- J L, two scalar Potter updates (y then z).
 //
 // Work mapping: a persistent grid; each warp takes work items of up to 32 tracks
-// (WorkShape, internal.h) and fits one track per lane.  While a lane computes the steps
-// of the current chunk, the warp's asynchronous copies (cp.async) bring the
-// next `RPS` clusters of all 32 tracks into the other half of a shared-memory
-// double buffer.  The alignment table and the geometry live in shared memory.
+// (WorkShape, internal.h) and fits one track per lane.  While a lane computes the
+// steps of the current chunk, its asynchronous copies (cp.async) bring the next
+// `RPS` clusters of its track into a ring of windows in shared memory.  The
+// alignment table and the geometry live in shared memory.
 // Tracks are taken in an order that puts tracks of equal length into the same
 // warp (length_order.cu) so that a warp's lanes finish together.
 //
@@ -194,6 +194,10 @@ __device__ __forceinline__ void load_tables(const GeoRef& G, SmemTables& t) {
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gmem_src) : "memory");
 }
 // 16 bytes (L2 only, no L1 allocation).
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
@@ -645,46 +649,55 @@ struct TrackState {
   int used;
 };
 
-// Double-buffered staging of RPS clusters for each of a warp's 32 tracks.  Row
-// pitch RPS + 1 keeps the consumer's reads (lane t reads row t) conflict-free.
-// rowsec travels as the aligned 32-bit word that contains it.
+// Staging of a warp's clusters: each lane copies its own track's, in windows of 4
+// clusters aligned in memory (three asynchronous copies of 16, 16 and 8 bytes a
+// window), into a ring of windows; a step reads its cluster at its place in its
+// window.  No lane reads another's windows, so no shuffle hands tracks around and
+// nothing but the lane's own copies is waited for.  (Copies of single clusters,
+// each group of lanes taking consecutive ones of one track, cost about 38 of the
+// step's 340 instructions: shuffles, bounds of the rowsec words, three copies and
+// their addresses per cluster.)  y and z bypass L1, whose room the alignment tables
+// need.  A window that reaches beyond the arrays, or any window where the arrays
+// are not aligned, is copied cluster by cluster.  Plain fit of 400,000 tracks: 725
+// -> 657 us (666 through L1; 699 through L1 with a ring of 4 windows, whose shared
+// memory comes out of L1), recorded 980 -> 897.
 template <int RPS>
 struct WarpStage {
-  float y[2][kWarp][RPS + 1];
-  float z[2][kWarp][RPS + 1];
-  uint32_t rs[2][kWarp][RPS + 1];
+  static constexpr int kWindows = fit_stage_windows(RPS);
+  float4 y[kWindows][kWarp];
+  float4 z[kWindows][kWarp];
+  uint2 rs[kWindows][kWarp];
 };
 
-// Issue the copies of local steps [c0, c0 + RPS) of every lane's pass into
-// buffer b: lane t's step i is hit first_t + dir * i (valid for i < count_t).
-// Each group of RPS lanes copies RPS consecutive clusters of one track.
+// The windows of one lane's pass: step i is hit first + dir i, window r is
+// (first >> 2) + dir r, and `last` the largest r that holds a step.
+struct LaneWindows {
+  int base, dir, last;
+};
+
+__device__ __forceinline__ bool windows_aligned(const FitArgs& a) {
+  return (((uintptr_t)a.y | (uintptr_t)a.z) & 15u) == 0 && ((uintptr_t)a.rowsec & 7u) == 0;
+}
+
 template <int RPS>
-__device__ __forceinline__ void stage_issue(WarpStage<RPS>& st, int b, const FitArgs& a, int my_first,
-                                            int my_count, int dir, int c0, int lane) {
-  const uintptr_t rs_begin = (uintptr_t)a.rowsec;
-  const uintptr_t rs_end = (uintptr_t)(a.rowsec + a.n_hits);
-#pragma unroll
-  for (int it = 0; it < RPS; ++it) {
-    const int e = it * kWarp + lane;
-    const int t = e / RPS;
-    const int k = e % RPS;
-    const int first_t = __shfl_sync(0xffffffffu, my_first, t);
-    const int count_t = __shfl_sync(0xffffffffu, my_count, t);
-    const int i = c0 + k;
-    if (i < count_t) {
-      const int h = first_t + dir * i;
-      cp_async4(&st.y[b][t][k], a.y + h);
-      cp_async4(&st.z[b][t][k], a.z + h);
-      const uint16_t* rp = a.rowsec + h;
-      const uintptr_t wa = (uintptr_t)rp & ~(uintptr_t)3;
-      if (wa >= rs_begin && wa + 4 <= rs_end) {
-        cp_async4(&st.rs[b][t][k], (const void*)wa);
-      } else {  // a cluster whose 32-bit word reaches outside the array
-        st.rs[b][t][k] = (uint32_t)__ldg(rp) << (16u * (unsigned)(((uintptr_t)rp >> 1) & 1u));
-      }
+__device__ __forceinline__ void stage_window(WarpStage<RPS>& st, const FitArgs& a, const LaneWindows& L, int r,
+                                             bool aligned, int lane) {
+  if (r > L.last) return;
+  const int slot = (unsigned)r % (unsigned)WarpStage<RPS>::kWindows;
+  const int h = (L.base + L.dir * r) * 4;
+  if (aligned && (int64_t)h + 4 <= a.n_hits) {
+    cp_async16(&st.y[slot][lane], a.y + h);
+    cp_async16(&st.z[slot][lane], a.z + h);
+    cp_async8(&st.rs[slot][lane], a.rowsec + h);
+  } else {
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+      if ((int64_t)h + k >= a.n_hits) break;
+      cp_async4(reinterpret_cast<float*>(&st.y[slot][lane]) + k, a.y + h + k);
+      cp_async4(reinterpret_cast<float*>(&st.z[slot][lane]) + k, a.z + h + k);
+      reinterpret_cast<uint16_t*>(&st.rs[slot][lane])[k] = __ldg(a.rowsec + h + k);
     }
   }
-  cp_async_commit();
 }
 
 struct BlockSmem {
@@ -796,7 +809,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
   const SmemTables& T = B.T;
   const int lane = threadIdx.x & 31;
   WarpStage<RPS>& st = stages[threadIdx.x >> 5];
-  const unsigned rs_par0 = (unsigned)(((uintptr_t)a.rowsec >> 1) & 1u);
+  const bool aligned = windows_aligned(a);
   const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
 
 #pragma unroll 1
@@ -890,26 +903,28 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) count_max = max(count_max, __shfl_xor_sync(0xffffffffu, count_max, o));
       if (count_max == 0) continue;
-      __syncwarp();
-      stage_issue<RPS>(st, 0, a, my_first, my_count, dir, 0, lane);
-      int buf = 0;
+      constexpr int kRefill = RPS / 4;  // windows
+      LaneWindows L;
+      L.base = my_first >> 2;
+      L.dir = dir;
+      L.last = my_count > 0 ? dir * (((my_first + dir * (my_count - 1)) >> 2) - L.base) : -1;
+#pragma unroll
+      for (int r = 0; r <= kRefill; ++r) stage_window<RPS>(st, a, L, r, aligned, lane);
+      cp_async_commit();
 #pragma unroll 1
       for (int c0 = 0; c0 < count_max; c0 += RPS) {
-        const bool more = c0 + RPS < count_max;
-        if (more) {
-          stage_issue<RPS>(st, buf ^ 1, a, my_first, my_count, dir, c0 + RPS, lane);
-          cp_async_wait<1>();
-        } else {
-          cp_async_wait<0>();
-        }
-        __syncwarp();
+        // the windows of the refill after this one
+#pragma unroll
+        for (int r = 1; r <= kRefill; ++r) stage_window<RPS>(st, a, L, c0 / 4 + kRefill + r, aligned, lane);
+        cp_async_commit();
+        cp_async_wait<1>();
 #pragma unroll 1
         for (int k = 0; k < RPS; ++k) {
           const int i = c0 + k;
           if (!go || i >= my_count) continue;
           const int h = my_first + dir * i;
-          const unsigned shift = 16u * ((rs_par0 + (unsigned)h) & 1u);
-          const int rsv = (int)((st.rs[buf][lane][k] >> shift) & 0xffffu);
+          const int slot = (unsigned)(dir * ((h >> 2) - L.base)) % (unsigned)WarpStage<RPS>::kWindows;
+          const int rsv = (int)reinterpret_cast<const uint16_t*>(&st.rs[slot][lane])[h & 3];
           const int row = rsv >> 6;
           const int sec = rsv & 63;
           if (row >= G.n_rows || sec >= kNSectors) {
@@ -920,8 +935,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
           }
           const float2 d = FRAMES ? reinterpret_cast<const float2*>(lane_align)[sec * kMaxRows + row]
                                   : reinterpret_cast<const float2*>(B.align)[sec * kMaxRows + row];
-          const float m0 = st.y[buf][lane][k] - d.x;
-          const float m1 = st.z[buf][lane][k] - d.y;
+          const float m0 = reinterpret_cast<const float*>(&st.y[slot][lane])[h & 3] - d.x;
+          const float m1 = reinterpret_cast<const float*>(&st.z[slot][lane])[h & 3] - d.y;
           const int sec18 = side_sector(sec);
           if (RECORD == 2 && on_tape) {
             if (FORM == 1) {
@@ -997,8 +1012,6 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
           S.used += 1;
           if (pass == 0) last = i;
         }
-        __syncwarp();
-        buf ^= 1;
       }
     }
 

@@ -186,11 +186,15 @@ constexpr unsigned long long kErrRowSector = 2;
 constexpr unsigned long long kErrTimeout = 3;
 
 // Shared memory of a fit block (geometry tables + alignment table) and of one
-// warp's double-buffered cluster staging with `rps` clusters per refill: the
-// host sizes the launch of a kernel compiled at run time with these.
+// warp's cluster staging with `rps` clusters per refill: the host sizes the launch
+// of a kernel compiled at run time with these.
 constexpr int kTablesFloats = kMaxRows + 2 * kNSide * kNSide;
 constexpr int kFitBlockSmemBytes = 4 * (kTablesFloats + kAlignFloats);
-__host__ __device__ constexpr int fit_warp_stage_bytes(int rps) { return 3 * 2 * kWarp * (rps + 1) * 4; }
+// A warp's staging: `fit_stage_windows` aligned windows of 4 clusters (y 16 B, z 16 B,
+// rowsec 8 B) for each of its 32 tracks, enough for the clusters of a refill at any
+// phase (rps / 4 + 1 windows) and those of the next one on their way.
+__host__ __device__ constexpr int fit_stage_windows(int rps) { return 2 * (rps / 4) + 1; }
+__host__ __device__ constexpr int fit_warp_stage_bytes(int rps) { return fit_stage_windows(rps) * kWarp * 40; }
 // Blocks per SM the fit asks for (__launch_bounds__) at each supported shape.
 __host__ __device__ constexpr int fit_min_blocks(int rps, int warps) { return (rps == 4 && warps == 24) || rps == 16 || warps == 16 ? 1 : 2; }
 

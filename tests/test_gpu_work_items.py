@@ -118,3 +118,29 @@ def test_items_without_room_on_the_tape_leave_checkpoints(mode):
             a, b = a.double(), b.double()
             assert torch.equal(torch.isnan(a), torch.isnan(b))
             assert float((a - b).nan_to_num().norm()) <= 1e-5 * float(a.nan_to_num().norm())
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3, 4])
+@pytest.mark.parametrize("det", [False, True], ids=["fast", "det"])
+def test_clusters_at_any_alignment(pool, shift, det):
+    # the clusters of 700 tracks begin `shift` elements into their arrays, which end
+    # with the last cluster: windows of 4 are whole, cut off at the end, or (not a
+    # multiple of 4 elements) not aligned at all; in the middle of the arrays they
+    # reach into the neighbouring tracks
+    fr, _ = pool
+    full, _, _ = _repeat(fr, POOL)
+
+    def moved(t):
+        big = torch.zeros(t.numel() + shift, dtype=t.dtype, device="cuda")
+        big[shift:] = t
+        return big[shift:]
+
+    dev = dict(full, y=moved(full["y"]), z=moved(full["z"]), rowsec=moved(full["rowsec"]))
+    f = tf.Fitter(fr.geometry, fr.bz, deterministic=det)
+    try:
+        a, b = f.fit(full), f.fit(dev)
+        assert f.status()[0] == tf.OK
+        for k in ("params", "cov", "chi2", "ndf"):
+            assert torch.equal(_bits(a[k]), _bits(b[k])), k
+    finally:
+        f.close()
