@@ -740,7 +740,7 @@ def main():
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "roofline": {"bound": "alu", "achieved": bwd_f["achieved_method"], "peak": peak_tf, "unit": "TFLOP/s",
                      "frac": bwd_f["frac_method"], "traffic": _traffic("backward_" + args.mode),
-                     "kernel": "backward_kernel", "launch_ms": bwd_ms,
+                     "kernel": "tape_reverse_ud_kernel", "launch_ms": bwd_ms,
                      "frac_impl": bwd_f["frac_impl"], "achieved_impl": bwd_f["achieved_impl"],
                      "count": "achieved/frac: method count (480 flop per cluster for the fit, x2.5 for the reverse); "
                               "*_impl: the form as implemented (flops.py; fast mode: U-D)",
@@ -751,7 +751,7 @@ def main():
                       "traffic": _traffic("fit_" + args.mode)},
         "hits_per_s": value * mhits,
         "e2e": e2e,
-        "gpu_launches": 4 * args.steps,
+        "gpu_launches": 5 * args.steps,
         "clocks": clocks,
         "config": {"workload": WORKLOAD, "step": "fit with checkpoints + adjoint (gradients w.r.t. alignment and seeds)",
                    "mode": args.mode, "tracks": fr.n_tracks, "hits": fr.n_hits, "mean_hits_per_track": mhits,

@@ -23,7 +23,8 @@ struct Resident {
 };
 template <class K>
 cudaError_t resident_blocks(K kernel, int threads, size_t smem, Resident& r) {
-  if (r.blocks != 0) return cudaSuccess;
+  // (several threads may come here at once: blocks is the last to be written)
+  if (__atomic_load_n(&r.blocks, __ATOMIC_ACQUIRE) != 0) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
@@ -33,7 +34,7 @@ cudaError_t resident_blocks(K kernel, int threads, size_t smem, Resident& r) {
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   r.sms = sms;
-  r.blocks = sms * per_sm;
+  __atomic_store_n(&r.blocks, sms * per_sm, __ATOMIC_RELEASE);
   return cudaSuccess;
 }
 

@@ -124,6 +124,7 @@ struct tpcfit_handle {
   int64_t tape_item_cap = 0;
   bool rec_tape = false;       // the recorded fit wrote the tape, with every
   int rec_every = 1;           //   rec_every-th state (U-D form)
+  bool rec_sorted = false;     // its work items follow d_perm
   float* d_gm = nullptr;
   int64_t gm_cap = 0;          // floats
   unsigned char* d_keys = nullptr;
@@ -173,7 +174,7 @@ tpcfit_status ensure_pipe(tpcfit_handle* h) {
 // Room for the tape of a recorded fit (kernel_abi.h) and its shape; without one
 // (a.tape null) the fit leaves checkpoints: another form of fit, no memory, or a
 // tape of more than half of what is free.
-void ensure_tape(tpcfit_handle* h, FitArgs& a) {
+void ensure_tape(tpcfit_handle* h, FitArgs& a, cudaStream_t s) {
   const bool ud = a.form == 1;
   if (h->lanes_per_track != 1 || !(h->deterministic || a.mat || ud)) return;
   const int64_t T = item_tracks(a.n_tracks, h->sms);
@@ -190,6 +191,11 @@ void ensure_tape(tpcfit_handle* h, FitArgs& a) {
                                          : items * tape_rows(ud, kMaxRows, every);
   if (rows > INT32_MAX) return;
   const int64_t need = rows * T;
+  if (need > h->tape_cap || items > h->tape_item_cap) {
+    // nothing is allocated while the stream is being captured
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return;
+  }
   if (need > h->tape_cap) {
     size_t avail = 0, total = 0;
     if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
@@ -212,13 +218,24 @@ void ensure_tape(tpcfit_handle* h, FitArgs& a) {
   a.tape_every = every;
 }
 
+// Room for the length permutation; a recording follows the present one, so its
+// contents stay.
 tpcfit_status ensure_perm(tpcfit_handle* h, int64_t n) {
   if (n <= h->perm_cap) return TPCFIT_OK;
-  if (h->d_perm) cudaFree(h->d_perm);
-  h->d_perm = nullptr;
-  h->perm_cap = 0;
-  cudaError_t e = cudaMalloc(&h->d_perm, sizeof(int32_t) * (size_t)n);
+  int32_t* p = nullptr;
+  cudaError_t e = cudaMalloc(&p, sizeof(int32_t) * (size_t)n);
   if (e != cudaSuccess) return from_cuda(e);
+  if (h->d_perm) {
+    e = cudaDeviceSynchronize();
+    if (e == cudaSuccess)
+      e = cudaMemcpy(p, h->d_perm, sizeof(int32_t) * (size_t)h->perm_cap, cudaMemcpyDeviceToDevice);
+    if (e != cudaSuccess) {
+      cudaFree(p);
+      return from_cuda(e);
+    }
+    cudaFree(h->d_perm);
+  }
+  h->d_perm = p;
   h->perm_cap = n;
   return TPCFIT_OK;
 }
@@ -387,7 +404,8 @@ tpcfit_status tpcfit_fit(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
     a.ck_last = h->d_ck_last;
     a.ck_slots = slots;
     h->ck_slots = slots;
-    ensure_tape(h, a);
+    ensure_tape(h, a, s);
+    h->rec_sorted = h->sort_by_length != 0;
     h->rec_tape = a.tape != nullptr;
     h->rec_every = a.tape_every;
   }
@@ -589,7 +607,7 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
   b.off = track_offsets;
   b.n_tracks = n_tracks;
   b.align = h->d_align;
-  b.perm = h->sort_by_length ? h->d_perm : nullptr;
+  b.perm = h->rec_sorted ? h->d_perm : nullptr;
   b.ndf = ndf;
   b.ck = h->d_ck;
   b.ck_last = h->d_ck_last;
@@ -688,7 +706,7 @@ tpcfit_status run_smooth(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
   a.off = track_offsets;
   a.n_tracks = n_tracks;
   a.align = h->d_align;
-  a.perm = h->sort_by_length ? h->d_perm : nullptr;
+  a.perm = h->rec_sorted ? h->d_perm : nullptr;
   a.ndf = ndf;
   a.ck = h->d_ck;
   a.ck_last = h->d_ck_last;

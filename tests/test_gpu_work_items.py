@@ -144,3 +144,25 @@ def test_clusters_at_any_alignment(pool, shift, det):
             assert torch.equal(_bits(a[k]), _bits(b[k])), k
     finally:
         f.close()
+
+
+def test_the_recording_outlives_other_settings(pool):
+    # the adjoint follows the recorded fit's order of the tracks, whatever the sort
+    # switch and the reserved size are by then
+    fr, _ = pool
+    dev, _, _ = _repeat(fr, POOL)
+    g = torch.ones(POOL, device="cuda")
+    f = tf.Fitter(fr.geometry, fr.bz, deterministic=True)
+    try:
+        f.set_record(True)
+        out = f.fit(dev)
+        ga, gs = f.backward(dev, out, g)
+        sm = f.smooth(dev, out)["chi2"]
+        f.set_config(sort_by_length=False)
+        tf.tpcfit_reserve(f.h, 3_000_000)
+        ga2, gs2 = f.backward(dev, out, g)
+        sm2 = f.smooth(dev, out)["chi2"]
+        assert torch.equal(_bits(ga), _bits(ga2)) and torch.equal(_bits(gs), _bits(gs2))
+        assert torch.equal(_bits(sm), _bits(sm2))
+    finally:
+        f.close()
