@@ -1,7 +1,7 @@
 """Alignment recovery: fit + adjoint + Adam on the 36 x 152 x 2 offsets, on the device.
 
 Each iteration uploads the current offset estimate to the fitter, fits every
-track with checkpoints, runs the adjoint of L = mean chi2 over fitted tracks
+track with recording, runs the adjoint of L = mean chi2 over fitted tracks
 and applies one Adam step (Kingma & Ba, 2015) to the offsets.  The iteration
 is captured in a CUDA graph once and replayed.  The loop's state (offsets,
 Adam moments, step count) can be written to a file every few iterations and

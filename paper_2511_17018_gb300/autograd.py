@@ -1,7 +1,7 @@
 """torch.autograd.Function over the library's fit and its hand-written adjoint.
 
 chi2 = TpcFit.apply(alignment, seeds, fitter, dev) runs tpcfit_fit with
-checkpoint recording; backward calls tpcfit_fit_backward with grad_chi2 =
+recording; backward calls tpcfit_fit_backward with grad_chi2 =
 dL/dchi2 and returns dL/dalignment [36,152,2] and dL/dseeds [5,N].  Tracks
 that fail (ndf <= 0) have chi2 = NaN in the output; mask them before summing.
 """

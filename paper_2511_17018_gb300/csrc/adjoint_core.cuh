@@ -8,12 +8,16 @@
 // and dL/dseed_i.  The outward pass feeds the inward one through its final
 // state (the covariance is reset, the outward chi2 is not part of L).
 //
-// Checkpoints: the forward writes the filter state (p, L, x, sector)
-// before every kCkptEvery-th step of each pass.  The backward walks the
+// Tape: the forward leaves the filter states of both passes on a tape, laid out
+// so that a warp reads a state of its 32 tracks as contiguous rows, and the
+// backward reverses the steps one by one from it (recomputing each step's
+// intermediates from the state before it).
+//
+// Checkpoints, where there is no place on the tape: the forward writes the filter
+// state before every kCkptEvery-th step of each pass.  The backward walks the
 // segments of a track in reverse: it recomputes a segment's steps from its
-// checkpoint into a per-warp segment store, then reverses the steps one by one
-// (recomputing each step's intermediates from the state before it).  States carry y and z
-// as residuals from the current cluster's measurement, like the fit.
+// checkpoint into a per-warp segment store, then reverses them.  States carry y and
+// z as residuals from the current cluster's measurement, like the fit.
 #pragma once
 
 namespace tpcfit {

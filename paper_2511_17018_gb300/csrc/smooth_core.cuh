@@ -15,8 +15,8 @@
 //
 // Both predictions follow from states that the recorded fit left on its tape, so
 // the clusters of a track are smoothed independently of each other
-// (smooth_tape_kernel).  Items without a place on the tape go through
-// smooth_kernel, from the checkpoints:
+// (smooth_tape_kernel).  Items without a place on the tape, and the last clusters
+// of some of the others, go through smooth_kernel.  From the checkpoints:
 //
 // Work mapping of smooth_kernel: the outward filter runs forward from the seed, cluster by
 // cluster.  The inward predictions are needed in the same order, which is the
@@ -243,13 +243,23 @@ constexpr size_t smooth_smem_bytes() {
 // (a.state, a.state_cov); without it the kernel carries none of that code.
 //
 // After a fit that left a U-D tape it does two things.  Items without a place on
-// the tape go through it whole.  Of the others it smooths the states of the last
-// kSmoothEnds clusters of each track, whose covariance depends on rounding at 3e-5
-// in norm (the inward prior is diffuse there: a cluster or two against 100 cm^2
-// and steep tracks): they keep the square-root sequence, along the outward filter
-// from the seed, and smooth_tape_kernel does the rest (30,000 tracks: 169 us for
-// the ends, 185 for the rest).
+// the tape go through it whole.  Of the others it smooths the last kSmoothEnds
+// clusters, the ends, where the outputs depend on rounding: at steep angles
+// (|sin phi| towards 1) a filter amplifies it, and the inward prior is diffuse
+// there.  They keep the square-root sequence, along the outward filter from the
+// seed, and smooth_tape_kernel does the rest.  The states' covariance depends on it
+// at 3e-5 in norm, so every track's end is smoothed here (30,000 tracks: 169 us for
+// the ends, 185 for the rest).  The residuals do in single elements only (1e-3 of
+// the largest, and 3e-4 below |sin phi| = 0.9), so only the steep tracks' ends are,
+// gathered by each warp from its share of the tracks.
 constexpr int kSmoothEnds = kCkptEvery;
+constexpr float kSmoothSteep = 0.9f;
+
+// |sin phi| next to the end of a track of `steps` steps above kSmoothSteep; its
+// outward states from row0 on.
+__device__ __forceinline__ bool steep_end(const float4* row0, int steps, int every, int pitch) {
+  return fabsf(__ldg(row0 + kUDRows * ((steps - 1) / every) * pitch).z) > kSmoothSteep;
+}
 
 // An outward or inward pass's first state from the U-D tape, as a checkpoint.
 __device__ __forceinline__ void tape_first_state(const float4* src, int pitch, StepState& S) {
@@ -267,11 +277,14 @@ __device__ __forceinline__ void tape_first_state(const float4* src, int pitch, S
   unpack_state(v, S);
 }
 
+constexpr int kMaxShare = kStateF4 * kWarp * 4;  // tracks that a warp's list holds
+
 template <int WARPS, bool MAT, bool STATES>
 __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_constant__ SmoothArgs a) {
   const GeoRef& G = a.geo;
-  const bool ends_too = STATES && a.ck_form == 1;
-  if (a.tape_item && !ends_too && a.work[kWorkMissing] == 0) return;
+  const bool ends_too = a.tape_item && a.ck_form == 1;
+  const bool missing = !a.tape_item || a.work[kWorkMissing] > 0;
+  if (!ends_too && !missing) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdSmem& B = *reinterpret_cast<BwdSmem*>(smem_raw);
   load_block_tables(G, B.T, B.align, a.align);
@@ -281,15 +294,54 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
   BwdWarpBufs& W = reinterpret_cast<BwdWarpBufs*>(smem_raw + sizeof(BwdSmem))[warp];
   float4* const gs = a.seg + ((int64_t)blockIdx.x * WARPS + warp) * (kCkptEvery * kStateF4 * kWarp) + lane;
   const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
+  // residuals: after the items (none if all are on the tape) the tracks once more,
+  // `share` of them at a time, for the steep ones' ends
+  const bool gather = !STATES && ends_too;
+  const int n_warps = gridDim.x * (blockDim.x >> 5);
+  const int share = min(kMaxShare, ((a.n_tracks + n_warps - 1) / n_warps + kWarp - 1) / kWarp * kWarp);
+  const int64_t lists = gather ? ((int64_t)a.n_tracks + share - 1) / share : 0;
+  const int64_t items = STATES || missing ? n_items : 0;
+  int* const list = reinterpret_cast<int*>(&W.ck[0][0]);  // no checkpoint is read for the ends
+  int listed = 0, taken = 0;
 #pragma unroll 1
-  for (bool first = true;; first = false) {
-    const int64_t item = next_item(a.work, n_items, first);
-    if (item < 0) break;
-    const int2 place = a.tape_item ? a.tape_item[item] : make_int2(-1, 0);
-    const bool ends = ends_too && place.x >= 0;
+  for (bool first = true;;) {
+    int64_t item = -1;
+    if (taken >= listed) {
+      const int64_t unit = next_item(a.work, items + lists, first);
+      first = false;
+      if (unit < 0) break;
+      if (unit < items) {
+        item = unit;
+      } else {
+        const int64_t slot0 = (unit - items) * share;
+        listed = taken = 0;
+        __syncwarp();
+#pragma unroll 1
+        for (int64_t k = slot0 + lane; k - lane < min(slot0 + share, (int64_t)a.n_tracks); k += kWarp) {
+          bool steep = false;
+          if (k < a.n_tracks) {
+            const int32_t t = a.perm ? a.perm[k] : (int32_t)k;
+            const int2 at = a.tape_item[k / a.item_tracks];
+            if (at.x >= 0 && a.ndf[t] > 0)
+              steep = steep_end(tape_row0(a.tape, at, a.item_tracks, (int)(k % a.item_tracks)) + at.y * a.item_tracks,
+                                a.ck_last[t] + 1, a.tape_every, a.item_tracks);
+          }
+          const unsigned m = __ballot_sync(0xffffffffu, steep);
+          if (steep) list[listed + __popc(m & ((1u << lane) - 1))] = (int)k;
+          listed += __popc(m);
+        }
+        __syncwarp();
+        if (listed == 0) continue;
+      }
+    }
+    const bool from_list = item < 0;
+    const int64_t slot = from_list ? (taken + lane < listed ? list[taken + lane] : a.n_tracks) : item * a.item_tracks + lane;
+    const bool have = (from_list || lane < a.item_tracks) && slot < a.n_tracks;
+    if (from_list) taken += kWarp;
+    const int2 place = a.tape_item && (have || !from_list) ? a.tape_item[from_list ? slot / a.item_tracks : item]
+                                                           : make_int2(-1, 0);
+    const bool ends = from_list || (STATES && ends_too && place.x >= 0);
     if (place.x >= 0 && !ends) continue;  // smooth_tape_kernel's
-    const int64_t slot = item * a.item_tracks + lane;
-    const bool have = lane < a.item_tracks && slot < a.n_tracks;
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
     const int begin = have ? a.off[trk] : 0;
     const bool fitted = have && a.ndf[trk] > 0;
@@ -297,7 +349,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
     const int last = steps - 1;
     if (have && !ends) write_nan_clusters(a, begin + steps, a.off[trk + 1]);  // without an estimate
     const int64_t slot0 = (begin >> kCkptShift) + trk;
-    const float4* const row0 = ends ? tape_row0(a.tape, place, a.item_tracks, lane) + place.y * a.item_tracks : nullptr;
+    const float4* const row0 = ends && have ? tape_row0(a.tape, place, a.item_tracks, (int)(slot % a.item_tracks)) +
+                                                  place.y * a.item_tracks
+                                            : nullptr;
     // outward filter: from its first state (the seed, factor L0)
     StepState O;
     float omy = 0.0f, omz = 0.0f;  // measurement O's residuals refer to (none for the seed)
@@ -418,7 +472,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
           transport(O.L, J);
           if (MAT) material_factor(O.L, N);
         }
-        if (a.resid) {
+        if (a.resid && combine) {
           float r[2], R[3], c2;
           smooth_combine(G, po, O.L, pi, SI.L, r, R, c2);
           reinterpret_cast<float2*>(a.resid)[h] = make_float2(r[0], r[1]);
@@ -536,7 +590,8 @@ __device__ __forceinline__ void combine_ud(float p[5], float u[10], float d[5], 
 // cluster are two turns of one loop, since two copies of the prediction and the
 // recomputed step miss the instruction cache (1.4 warps waiting for instructions
 // per issue, 0.3 as a loop).  Measured: leave-one-out residuals of 100,000 tracks
-// 823 -> 465 us, smoothed states of 30,000 tracks, the ends included, 675 -> 358 us.
+// 823 -> 593 us (465 without the steep tracks' ends, whose one chain of steps a warp
+// is serial), smoothed states of 30,000 tracks, the ends included, 675 -> 363 us.
 // The unit's clusters are copied into shared memory once and each state one turn
 // ahead; the outputs leave through shared memory too, a track's run of clusters at
 // a time instead of single words.
@@ -615,11 +670,14 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_tape_kernel(const __grid
     const bool fitted = have && a.ndf[trk] > 0;
     const int steps = fitted ? a.ck_last[trk] + 1 : 0;
     if (have && part == 0) write_nan_clusters(a, begin + steps, a.off[trk + 1]);  // without an estimate
-    // the states of a track's last clusters are smooth_kernel's (U-D form)
-    const int upto = STATES && FORM == 1 ? max(0, steps - kSmoothEnds) : steps;
-    const int most = __reduce_max_sync(0xffffffffu, upto);
     const float4* const row0 = tape_row0(a.tape, place, pitch, lane);
     const int every = FORM == 1 ? a.tape_every : 1;
+    // the last clusters are smooth_kernel's (U-D form: all tracks' states, the steep
+    // ones' residuals)
+    int upto = steps;
+    if (FORM == 1 && steps > 0 && (STATES || steep_end(row0 + place.y * pitch, steps, every, pitch)))
+      upto = max(0, steps - kSmoothEnds);
+    const int most = __reduce_max_sync(0xffffffffu, upto);
     const int states = (int)tape_states(place.y, every);
 
     // a track's cluster: measured (y, z), the row's x, sector mod 18
@@ -876,6 +934,10 @@ inline cudaError_t smooth_store(int64_t& float4s) {
 
 template <bool MAT, bool STATES>
 cudaError_t launch_smooth_cfg(const SmoothArgs& a, cudaStream_t s) {
+  if (!STATES && a.tape && a.ck_form == 1) {  // it may count items and lists
+    const cudaError_t e = clear_work(a.work, false, true, s);
+    if (e != cudaSuccess) return e;
+  }
   return launch_persistent(smooth_kernel<kSmoothWarps, MAT, STATES>, smooth_resident<MAT, STATES>(), kSmoothWarps,
                            sizeof(BwdSmem), sizeof(BwdWarpBufs), a, s);
 }
@@ -916,7 +978,8 @@ cudaError_t launch_smooth_of(const SmoothArgs& a, cudaStream_t s) {
 #endif
     if (e != cudaSuccess) return e;
   }
-  // from checkpoints: everything, or the items that the tape had no room for
+  // from checkpoints: everything, or the items that the tape had no room for; and
+  // the ends
   return a.mat ? launch_smooth_cfg<true, STATES>(a, s) : launch_smooth_cfg<false, STATES>(a, s);
 }
 

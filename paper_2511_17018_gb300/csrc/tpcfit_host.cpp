@@ -630,8 +630,9 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
     b.tape_item = h->d_tape_item;
     b.tape_every = h->rec_every;
   }
-  // from checkpoints, one kernel recomputes each segment into a per-warp segment
-  // store that stays in L2 until the reverse reads it back
+  // for what is not on the tape, the kernels recompute each segment from its
+  // checkpoint into a per-warp segment store that stays in L2 until the reverse
+  // reads it back
   int64_t need = 0;
   e = h->deterministic ? backward_store_det(h->bwd_warps, b.phys, b.form, need)
                        : backward_store_fast(h->bwd_warps, b.phys, b.form, need);

@@ -4,7 +4,7 @@
 //
 // The backward may recompute a segment in any factorisation of the same
 // covariance: the adjoint of the objective depends on the covariance, not on
-// its factor.  A segment starts from the fit's checkpoint: the U-D fit's
+// its factor.  From checkpoints, a segment starts from the fit's: the U-D fit's
 // (p, U, D) as they are, or the square-root fit's (p, L), whose rows,
 // orthogonalised with unit weights, give U and D.  That conversion needs no
 // reverse: the U-D factorisation of a covariance is unique, so the
