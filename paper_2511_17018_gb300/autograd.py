@@ -4,6 +4,8 @@ chi2 = TpcFit.apply(alignment, seeds, fitter, dev) runs tpcfit_fit with
 recording; backward calls tpcfit_fit_backward with grad_chi2 =
 dL/dchi2 and returns dL/dalignment [36,152,2] and dL/dseeds [5,N].  Tracks
 that fail (ndf <= 0) have chi2 = NaN in the output; mask them before summing.
+A fitter keeps one recording: run the backward before the next fit on the same
+fitter, or use a fitter each.
 """
 from __future__ import annotations
 

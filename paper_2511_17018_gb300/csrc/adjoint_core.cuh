@@ -380,6 +380,13 @@ __device__ __forceinline__ void sqrt_from_ud_ckpt(StepState& S) {
 }
 
 // One cluster as stored (y, z, packed row/sector), loaded ahead of its use.
+// Steps of a pass over a track that the recorded fit fitted, 0 for the others.  The
+// recording has the last word: of a track without a fit it holds no state and no
+// cluster, whatever the caller's ndf (another fit's, say) makes of it.
+__device__ __forceinline__ int recorded_steps(const int32_t* ndf, const int32_t* ck_last, int32_t trk) {
+  return ndf[trk] > 0 ? ck_last[trk] + 1 : 0;
+}
+
 struct HitRaw {
   float y, z;
   int rs;
@@ -980,11 +987,11 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
     if (lane >= a.item_tracks || slot >= N) continue;
     const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
     const float g = __ldg(a.grad_chi2 + trk);
-    const bool fitted = a.ndf[trk] > 0;
+    const int steps = recorded_steps(a.ndf, a.ck_last, trk);
     float b_p[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    if (fitted) {
+    if (steps > 0) {
       const int begin = a.off[trk];
-      const int last = a.ck_last[trk];
+      const int last = steps - 1;
       float b_L[5][5];         // FORM 0: adjoint of the square-root factor
       float b_u[10], b_d[5];   // FORM 1: adjoint of the U-D factor
 #pragma unroll 1
@@ -998,7 +1005,6 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
 #pragma unroll
         for (int c = 0; c < 5; ++c) b_d[c] = 0.0f;
         const float b_chi = pass == 1 ? g : 0.0f;
-        const int steps = last + 1;
         const int nseg = (steps + kCkptEvery - 1) / kCkptEvery;
         // hit index of step i of this pass
         const int h0 = pass == 0 ? begin : begin + last;
@@ -1195,10 +1201,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_ud_kernel(const __
     const int64_t slot = item * pitch + lane;
     const bool have = lane < pitch && slot < N;
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
-    const bool fitted = have && a.ndf[trk] > 0;
-    const float g = fitted ? __ldg(a.grad_chi2 + trk) : 0.0f;
+    const int steps = have ? recorded_steps(a.ndf, a.ck_last, trk) : 0;
+    const float g = steps > 0 ? __ldg(a.grad_chi2 + trk) : 0.0f;
     const int begin = have ? a.off[trk] : 0;
-    const int steps = fitted ? a.ck_last[trk] + 1 : 0;
     const int most = __reduce_max_sync(0xffffffffu, steps);
     const float4* const row0 = tape_row0(a.tape, place, pitch, lane);
     float b_p[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
@@ -1290,7 +1295,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_ud_kernel(const __
       cp_async_wait<0>();
     }
     if (!have) continue;
-    if (!fitted && a.grad_meas) {
+    if (steps == 0 && a.grad_meas) {
       const int end = a.off[trk + 1];
       for (int h = begin; h < end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
     }
@@ -1365,10 +1370,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __gri
     const int64_t slot = item * pitch + lane;
     const bool have = lane < pitch && slot < N;
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
-    const bool fitted = have && a.ndf[trk] > 0;
-    const float g = fitted ? __ldg(a.grad_chi2 + trk) : 0.0f;
+    const int steps = have ? recorded_steps(a.ndf, a.ck_last, trk) : 0;
+    const float g = steps > 0 ? __ldg(a.grad_chi2 + trk) : 0.0f;
     const int begin = have ? a.off[trk] : 0;
-    const int steps = fitted ? a.ck_last[trk] + 1 : 0;
     const int most = __reduce_max_sync(0xffffffffu, steps);
     float b_p[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 1
@@ -1451,7 +1455,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __gri
       // b_p carries over, b_L does not
     }
     if (!have) continue;
-    if (!fitted && a.grad_meas) {
+    if (steps == 0 && a.grad_meas) {
       const int end = a.off[trk + 1];
       for (int h = begin; h < end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
     }

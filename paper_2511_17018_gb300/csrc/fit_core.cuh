@@ -1023,9 +1023,10 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
 
     // ---- outputs at the track's own index
     if (!have) continue;
-    if (RECORD) a.ck_last[trk] = last;
+    const bool good = status == 0 && S.used >= 3;
+    if (RECORD) a.ck_last[trk] = good ? last : -1;
     const int64_t N = a.n_tracks;
-    if (status == 0 && S.used >= 3) {
+    if (good) {
       a.params[trk] = S.my + S.p[0];
       a.params[N + trk] = S.mz + S.p[1];
 #pragma unroll

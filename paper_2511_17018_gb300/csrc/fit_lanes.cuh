@@ -395,9 +395,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) fit_kernel_lanes(const __grid_c
     }
 
     // ---- outputs at the track's own index (all lanes take part in the sums)
-    if (RECORD && have && g == 0) a.ck_last[trk] = last;
     const int64_t N = a.n_tracks;
     const bool good = have && status == 0 && used >= 3;
+    if (RECORD && have && g == 0) a.ck_last[trk] = good ? last : -1;
     float cov[15];
     {
       int e = 0;

@@ -101,7 +101,8 @@ struct FitArgs {
   unsigned int* work;          // work-item counter (zeroed by the launcher)
   // checkpoint recording for the adjoint (null = off)
   float* ck;                   // [2][ck_slots][32] filter state before every kCkptEvery-th step of each pass
-  int32_t* ck_last;            // [n_tracks] index of the last cluster of the outward pass
+  int32_t* ck_last;            // [n_tracks] index of the last cluster of the outward pass; -1: not fitted, nothing of
+                               // the track is to be read from the recording
   int64_t ck_slots;            // slots per pass: n_hits / kCkptEvery + n_tracks + 1
   // or the tape (null = checkpoints)
   float4* tape;

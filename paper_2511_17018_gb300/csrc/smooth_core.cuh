@@ -322,9 +322,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
           if (k < a.n_tracks) {
             const int32_t t = a.perm ? a.perm[k] : (int32_t)k;
             const int2 at = a.tape_item[k / a.item_tracks];
-            if (at.x >= 0 && a.ndf[t] > 0)
-              steep = steep_end(tape_row0(a.tape, at, a.item_tracks, (int)(k % a.item_tracks)) + at.y * a.item_tracks,
-                                a.ck_last[t] + 1, a.tape_every, a.item_tracks);
+            const int n = recorded_steps(a.ndf, a.ck_last, t);
+            if (at.x >= 0 && n > 0)
+              steep = steep_end(tape_row0(a.tape, at, a.item_tracks, (int)(k % a.item_tracks)) + at.y * a.item_tracks, n,
+                                a.tape_every, a.item_tracks);
           }
           const unsigned m = __ballot_sync(0xffffffffu, steep);
           if (steep) list[listed + __popc(m & ((1u << lane) - 1))] = (int)k;
@@ -344,8 +345,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
     if (place.x >= 0 && !ends) continue;  // smooth_tape_kernel's
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
     const int begin = have ? a.off[trk] : 0;
-    const bool fitted = have && a.ndf[trk] > 0;
-    const int steps = fitted ? a.ck_last[trk] + 1 : 0;
+    const int steps = have ? recorded_steps(a.ndf, a.ck_last, trk) : 0;
     const int last = steps - 1;
     if (have && !ends) write_nan_clusters(a, begin + steps, a.off[trk + 1]);  // without an estimate
     const int64_t slot0 = (begin >> kCkptShift) + trk;
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
     HitRaw ahead{};  // the cluster after the one taken next
     float m0 = 0.0f, m1 = 0.0f;
     int row = 0, sec = 0;
-    if (fitted) {
+    if (steps > 0) {
       if (ends) {
         tape_first_state(row0, a.item_tracks, O);
       } else {
@@ -667,8 +667,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_tape_kernel(const __grid
     const bool have = lane < pitch && slot < a.n_tracks;
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
     const int begin = have ? a.off[trk] : 0;
-    const bool fitted = have && a.ndf[trk] > 0;
-    const int steps = fitted ? a.ck_last[trk] + 1 : 0;
+    const int steps = have ? recorded_steps(a.ndf, a.ck_last, trk) : 0;
     if (have && part == 0) write_nan_clusters(a, begin + steps, a.off[trk + 1]);  // without an estimate
     const float4* const row0 = tape_row0(a.tape, place, pitch, lane);
     const int every = FORM == 1 ? a.tape_every : 1;

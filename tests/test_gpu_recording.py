@@ -1,0 +1,85 @@
+"""What a recording holds, and for which tracks and clusters the adjoint and the
+smoother answer (run on a GB300 with -m gpu)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2511_17018_gb300 import synth  # noqa: E402
+from paper_2511_17018_gb300 import tpcfit as tf  # noqa: E402
+
+# name: deterministic, lanes per track, factor of the fast fit and reverse, material
+KINDS = {"fast": (False, 1, 1, False), "det": (True, 1, 1, False), "material": (False, 1, 1, True),
+         "fast_checkpoints": (False, 1, 0, False), "det_checkpoints": (True, 8, 1, False)}
+
+
+def _fitter(fr, kind):
+    det, lanes, form, material = KINDS[kind]
+    f = tf.Fitter(fr.geometry, fr.bz, deterministic=det)
+    f.set_config(lanes, 4, 24, True)
+    f.set_fit_form(form)
+    f.set_backward_form(form)
+    f.set_material(synth.TPC_GAS if material else None)
+    f.set_record(True)
+    return f
+
+
+def _bits(t):
+    return t.contiguous().view(torch.int32)
+
+
+class Guarded:
+    """A tensor of n elements in the middle of a larger one that has to stay as it is."""
+
+    def __init__(self, *shape, margin=1024):
+        n = int(np.prod(shape))
+        self.big = torch.full((n + 2 * margin,), 7.0, device="cuda")
+        self.t = self.big[margin:margin + n].view(*shape)
+        self.margin = margin
+
+    def intact(self):
+        m = self.margin
+        return bool((self.big[:m] == 7.0).all()) and bool((self.big[-m:] == 7.0).all())
+
+
+def _follow(f, dev, ndf):
+    """Adjoint, residuals and states of the recorded fit, into guarded outputs."""
+    n = dev["offsets"].numel() - 1
+    H = dev["y"].numel()
+    o = dict(ga=Guarded(36 * 152 * 2), gs=Guarded(5, n), gm=Guarded(H, 2), resid=Guarded(H, 2), rcov=Guarded(H, 3),
+             chi2=Guarded(H), state=Guarded(H, 5), state_cov=Guarded(H, 15))
+    args = (f.h, dev["y"], dev["z"], dev["rowsec"], dev["offsets"], ndf)
+    tf.tpcfit_fit_backward(*args, torch.ones(n, device="cuda"), o["ga"].t, o["gs"].t, o["gm"].t)
+    tf.tpcfit_smooth(*args, o["resid"].t, o["rcov"].t, o["chi2"].t)
+    tf.tpcfit_smooth_states(*args, o["state"].t, o["state_cov"].t)
+    torch.cuda.synchronize()
+    for k, v in o.items():
+        assert v.intact(), k
+    return {k: v.t for k, v in o.items()}
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_the_recording_decides_which_tracks_were_fitted(kind):
+    # another fit's ndf calls tracks fitted that the recorded fit could not start:
+    # the recording holds nothing of them, so they count as not fitted
+    fr = synth.generate(300, 61)
+    dev = tf.frame_to_device(fr)
+    bad = torch.arange(0, 300, 7, device="cuda")
+    unusable = dict(dev, seeds=dev["seeds"].clone())
+    unusable["seeds"][2, bad] = 0.9995
+    f = _fitter(fr, kind)
+    try:
+        ndf_other = f.fit(dev)["ndf"].clone()
+        out = f.fit(unusable)
+        assert bool((ndf_other[bad] > 0).all()) and bool((out["ndf"][bad] == -1).all())
+        got = _follow(f, unusable, torch.where(out["ndf"] > 0, out["ndf"], ndf_other))
+        want = _follow(f, unusable, out["ndf"])
+        assert bool((got["gs"][:, bad] == 0).all())
+        for k in want:
+            if k == "ga" and not KINDS[kind][0]:  # atomics: the order of the additions is free
+                assert float((got[k] - want[k]).norm()) <= 1e-5 * float(want[k].norm())
+            else:
+                assert torch.equal(_bits(got[k]), _bits(want[k])), k
+    finally:
+        f.close()
