@@ -380,11 +380,20 @@ __device__ __forceinline__ void sqrt_from_ud_ckpt(StepState& S) {
 }
 
 // One cluster as stored (y, z, packed row/sector), loaded ahead of its use.
-// Steps of a pass over a track that the recorded fit fitted, 0 for the others.  The
+// A track's clusters and the steps of a pass over it, 0 if it has no fit.  The
 // recording has the last word: of a track without a fit it holds no state and no
-// cluster, whatever the caller's ndf (another fit's, say) makes of it.
-__device__ __forceinline__ int recorded_steps(const int32_t* ndf, const int32_t* ck_last, int32_t trk) {
-  return ndf[trk] > 0 ? ck_last[trk] + 1 : 0;
+// cluster, whatever the caller's ndf (another fit's, say) makes of it.  The range is
+// empty for the offsets that the fit refuses, so no cluster outside the arrays is
+// touched.
+struct RecordedTrack {
+  int begin = 0, end = 0, steps = 0;
+};
+template <class A>
+__device__ __forceinline__ RecordedTrack recorded_track(const A& a, int32_t trk) {
+  RecordedTrack r;
+  track_range(a.off, trk, a.n_hits, r.begin, r.end);
+  r.steps = a.ndf[trk] > 0 ? min(a.ck_last[trk] + 1, r.end - r.begin) : 0;
+  return r;
 }
 
 struct HitRaw {
@@ -987,10 +996,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
     if (lane >= a.item_tracks || slot >= N) continue;
     const int32_t trk = a.perm ? a.perm[slot] : (int32_t)slot;
     const float g = __ldg(a.grad_chi2 + trk);
-    const int steps = recorded_steps(a.ndf, a.ck_last, trk);
+    const RecordedTrack track = recorded_track(a, trk);
+    const int begin = track.begin, steps = track.steps;
     float b_p[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     if (steps > 0) {
-      const int begin = a.off[trk];
       const int last = steps - 1;
       float b_L[5][5];         // FORM 0: adjoint of the square-root factor
       float b_u[10], b_d[5];   // FORM 1: adjoint of the U-D factor
@@ -1125,9 +1134,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
         // b_p carries over, b_L does not
       }
     } else if (a.grad_meas) {
-      const int begin = a.off[trk];
-      const int end = a.off[trk + 1];
-      for (int h = begin; h < end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
+      for (int h = begin; h < track.end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
     }
 #pragma unroll
     for (int c = 0; c < 5; ++c) a.grad_seeds[(int64_t)c * N + trk] = b_p[c];
@@ -1201,9 +1208,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_ud_kernel(const __
     const int64_t slot = item * pitch + lane;
     const bool have = lane < pitch && slot < N;
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
-    const int steps = have ? recorded_steps(a.ndf, a.ck_last, trk) : 0;
+    const RecordedTrack track = have ? recorded_track(a, trk) : RecordedTrack();
+    const int begin = track.begin, steps = track.steps;
     const float g = steps > 0 ? __ldg(a.grad_chi2 + trk) : 0.0f;
-    const int begin = have ? a.off[trk] : 0;
     const int most = __reduce_max_sync(0xffffffffu, steps);
     const float4* const row0 = tape_row0(a.tape, place, pitch, lane);
     float b_p[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
@@ -1296,8 +1303,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_ud_kernel(const __
     }
     if (!have) continue;
     if (steps == 0 && a.grad_meas) {
-      const int end = a.off[trk + 1];
-      for (int h = begin; h < end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
+      for (int h = begin; h < track.end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
     }
 #pragma unroll
     for (int c = 0; c < 5; ++c) a.grad_seeds[(int64_t)c * N + trk] = b_p[c];
@@ -1370,9 +1376,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __gri
     const int64_t slot = item * pitch + lane;
     const bool have = lane < pitch && slot < N;
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
-    const int steps = have ? recorded_steps(a.ndf, a.ck_last, trk) : 0;
+    const RecordedTrack track = have ? recorded_track(a, trk) : RecordedTrack();
+    const int begin = track.begin, steps = track.steps;
     const float g = steps > 0 ? __ldg(a.grad_chi2 + trk) : 0.0f;
-    const int begin = have ? a.off[trk] : 0;
     const int most = __reduce_max_sync(0xffffffffu, steps);
     float b_p[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 1
@@ -1456,8 +1462,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __gri
     }
     if (!have) continue;
     if (steps == 0 && a.grad_meas) {
-      const int end = a.off[trk + 1];
-      for (int h = begin; h < end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
+      for (int h = begin; h < track.end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
     }
 #pragma unroll
     for (int c = 0; c < 5; ++c) a.grad_seeds[(int64_t)c * N + trk] = b_p[c];

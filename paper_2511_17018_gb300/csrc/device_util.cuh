@@ -8,6 +8,16 @@
 
 namespace tpcfit {
 
+// Cluster range [b, e) of track t; false, and an empty range, if its offsets are
+// out of order or leave the cluster arrays.
+__device__ __forceinline__ bool track_range(const int32_t* off, int64_t t, int64_t n_hits, int32_t& b, int32_t& e) {
+  b = off[t];
+  e = off[t + 1];
+  if (b >= 0 && e >= b && (int64_t)e <= n_hits) return true;
+  b = e = 0;
+  return false;
+}
+
 // Frame of track `trk`: f with base[f] <= trk < base[f + 1] (base[0] = 0,
 // base[n_frames] = total tracks); -1 if trk lies outside the table.
 __device__ __forceinline__ int frame_of(const int64_t* base, int n_frames, int64_t trk) {

@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "device_util.cuh"
 #include "internal.h"
 
 namespace tpcfit {
@@ -24,21 +25,13 @@ constexpr int kWarpsPerBlock = 8;
 constexpr int kTracksPerBlock = 32;
 constexpr int kUnroll = 4;  // times 32 clusters in flight
 
-// Cluster range of track t, empty if the offsets are out of order or outside
-// the cluster arrays.
-__device__ __forceinline__ void track_range(const int32_t* off, int32_t t, int64_t n_hits, int32_t& b, int32_t& e) {
-  b = off[t];
-  e = off[t + 1];
-  if (b < 0 || e < b || (int64_t)e > n_hits) b = e = 0;
-}
-
 // The ranges of the block's tracks (empty beyond the last one).
 __device__ __forceinline__ void block_ranges(const int32_t* off, int32_t n_tracks, int64_t n_hits, int32_t (&rb)[kTracksPerBlock],
                                              int32_t (&re)[kTracksPerBlock]) {
   if (threadIdx.x < kTracksPerBlock) {
     const int64_t t = (int64_t)blockIdx.x * kTracksPerBlock + threadIdx.x;
     int32_t b = 0, e = 0;
-    if (t < n_tracks) track_range(off, (int32_t)t, n_hits, b, e);
+    if (t < n_tracks) track_range(off, t, n_hits, b, e);
     rb[threadIdx.x] = b;
     re[threadIdx.x] = e;
   }

@@ -215,7 +215,16 @@ __device__ __forceinline__ void smooth_state(const float p1[5], const float L1[5
     }
 }
 
-__device__ __forceinline__ void write_nan_clusters(const SmoothArgs& a, int h0, int h1) {
+// The clusters of a track without an estimate.  A track that reaches beyond the
+// arrays has none; those of its clusters that lie inside are written unless the
+// offsets after it come back (they may be other tracks' then).
+__device__ __forceinline__ void write_nan_clusters(const SmoothArgs& a, int32_t trk, const RecordedTrack& track) {
+  int h0 = track.begin + track.steps, h1 = track.end;
+  if (h1 == 0 && a.off[trk + 1] > a.n_hits && a.off[trk] >= 0 &&
+      (trk + 1 == a.n_tracks || a.off[trk + 2] >= a.off[trk + 1])) {
+    h0 = a.off[trk];
+    h1 = (int)a.n_hits;
+  }
   const float qnan = __int_as_float(0x7fc00000);
   for (int h = h0; h < h1; ++h) {
     if (a.resid) {
@@ -322,7 +331,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
           if (k < a.n_tracks) {
             const int32_t t = a.perm ? a.perm[k] : (int32_t)k;
             const int2 at = a.tape_item[k / a.item_tracks];
-            const int n = recorded_steps(a.ndf, a.ck_last, t);
+            const int n = recorded_track(a, t).steps;
             if (at.x >= 0 && n > 0)
               steep = steep_end(tape_row0(a.tape, at, a.item_tracks, (int)(k % a.item_tracks)) + at.y * a.item_tracks, n,
                                 a.tape_every, a.item_tracks);
@@ -344,10 +353,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_kernel(const __grid_cons
     const bool ends = from_list || (STATES && ends_too && place.x >= 0);
     if (place.x >= 0 && !ends) continue;  // smooth_tape_kernel's
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
-    const int begin = have ? a.off[trk] : 0;
-    const int steps = have ? recorded_steps(a.ndf, a.ck_last, trk) : 0;
+    const RecordedTrack track = have ? recorded_track(a, trk) : RecordedTrack();
+    const int begin = track.begin, steps = track.steps;
     const int last = steps - 1;
-    if (have && !ends) write_nan_clusters(a, begin + steps, a.off[trk + 1]);  // without an estimate
+    if (have && !ends) write_nan_clusters(a, trk, track);
     const int64_t slot0 = (begin >> kCkptShift) + trk;
     const float4* const row0 = ends && have ? tape_row0(a.tape, place, a.item_tracks, (int)(slot % a.item_tracks)) +
                                                   place.y * a.item_tracks
@@ -666,9 +675,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1) smooth_tape_kernel(const __grid
     const int64_t slot = item * pitch + lane;
     const bool have = lane < pitch && slot < a.n_tracks;
     const int32_t trk = have ? (a.perm ? a.perm[slot] : (int32_t)slot) : 0;
-    const int begin = have ? a.off[trk] : 0;
-    const int steps = have ? recorded_steps(a.ndf, a.ck_last, trk) : 0;
-    if (have && part == 0) write_nan_clusters(a, begin + steps, a.off[trk + 1]);  // without an estimate
+    const RecordedTrack track = have ? recorded_track(a, trk) : RecordedTrack();
+    const int begin = track.begin, steps = track.steps;
+    if (have && part == 0) write_nan_clusters(a, trk, track);
     const float4* const row0 = tape_row0(a.tape, place, pitch, lane);
     const int every = FORM == 1 ? a.tape_every : 1;
     // the last clusters are smooth_kernel's (U-D form: all tracks' states, the steep

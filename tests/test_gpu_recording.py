@@ -83,3 +83,44 @@ def test_the_recording_decides_which_tracks_were_fitted(kind):
                 assert torch.equal(_bits(got[k]), _bits(want[k])), k
     finally:
         f.close()
+
+
+@pytest.mark.parametrize("where", ["last", "middle"])
+@pytest.mark.parametrize("kind", KINDS)
+def test_offsets_beyond_the_arrays_touch_nothing_outside(kind, where):
+    # an offset beyond the cluster arrays: the fit flags the tracks it bounds, the
+    # adjoint and the smoother leave everything outside the arrays alone and give
+    # the other tracks what they get with good offsets
+    fr = synth.generate(300, 62)
+    dev = tf.frame_to_device(fr)
+    H = fr.n_hits
+    at = 300 if where == "last" else 120
+    bad = [299] if where == "last" else [119, 120]
+    broken = dict(dev, offsets=dev["offsets"].clone())
+    for k in ("y", "z", "rowsec"):  # the arrays as views of larger ones
+        big = torch.zeros(H + 2048, dtype=dev[k].dtype, device="cuda")
+        big[1024:1024 + H] = dev[k]
+        broken[k] = big[1024:1024 + H]
+    broken["offsets"][at] = H + 5
+    keep = torch.ones(300, dtype=torch.bool, device="cuda")
+    keep[bad] = False
+    owner = torch.repeat_interleave(torch.arange(300, device="cuda"), (dev["offsets"][1:] - dev["offsets"][:-1]).long())
+    mine = keep[owner]
+    f = _fitter(fr, kind)
+    try:
+        want = _follow(f, dev, f.fit(dev)["ndf"])
+        assert f.status()[0] == tf.OK
+        out = f.fit(broken)
+        assert bool((out["ndf"][bad] == -2).all())
+        got = _follow(f, broken, out["ndf"])
+        st, code, trk = f.status()
+        assert st == tf.EDEVICE and code == 1 and trk in bad
+        assert torch.equal(_bits(got["gs"][:, keep]), _bits(want["gs"][:, keep]))
+        assert bool((got["gs"][:, bad] == 0).all())
+        for k in ("gm", "resid", "rcov", "chi2", "state", "state_cov"):
+            assert torch.equal(_bits(got[k][mine]), _bits(want[k][mine])), k
+        if where == "last":  # in order, but for the arrays' end
+            for k in ("resid", "rcov", "chi2", "state", "state_cov"):
+                assert bool(torch.isnan(got[k][~mine]).all()), k
+    finally:
+        f.close()
