@@ -288,7 +288,8 @@ tpcfit_status tpcfit_set_det_reduction(tpcfit_handle* h, int method);
  * Outputs (device, overwritten):
  *   grad_align: float [36][152][2], dL/d(dy, dz) of the alignment offsets;
  *   grad_seeds: float [5][n_tracks], dL/dseed;
- *   grad_meas:  float [n_hits][2], dL/d(measured y, z) per cluster, or NULL.
+ *   grad_meas:  float [n_hits][2], dL/d(measured y, z) per cluster, or NULL; 0
+ *               for the clusters that no step of a fitted track reached.
  * The backward runs the hand-written reverse of every step, copying the state
  * before each step into shared memory ahead of its use: from the recorded fit's
  * tape (with every second state on it, the others are recomputed one step at a

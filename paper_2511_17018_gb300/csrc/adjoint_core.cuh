@@ -915,7 +915,8 @@ __device__ __forceinline__ void red_add2(float* p, float v0, float v1) {
 }
 
 // prev: what the inward pass left at cluster h (read ahead by the caller; only
-// the outward pass, pass 0, adds to it).
+// the outward pass, pass 0, adds to it).  Clusters that no step of a fitted track
+// reached keep the zeros that the host put there.
 __device__ __forceinline__ void accumulate_meas_grad(const BwdArgs& a, int pass, int h, int row, int sec, float g0,
                                                      float g1, float2 prev) {
   if (a.grad_meas) {
@@ -1133,8 +1134,6 @@ __global__ void __launch_bounds__(WARPS * 32, 1) backward_kernel(const __grid_co
         // the inward pass starts from the outward result with the factor reset:
         // b_p carries over, b_L does not
       }
-    } else if (a.grad_meas) {
-      for (int h = begin; h < track.end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
     }
 #pragma unroll
     for (int c = 0; c < 5; ++c) a.grad_seeds[(int64_t)c * N + trk] = b_p[c];
@@ -1302,9 +1301,6 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_ud_kernel(const __
       cp_async_wait<0>();
     }
     if (!have) continue;
-    if (steps == 0 && a.grad_meas) {
-      for (int h = begin; h < track.end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
-    }
 #pragma unroll
     for (int c = 0; c < 5; ++c) a.grad_seeds[(int64_t)c * N + trk] = b_p[c];
   }
@@ -1461,9 +1457,6 @@ __global__ void __launch_bounds__(WARPS * 32, 1) tape_reverse_kernel(const __gri
       // b_p carries over, b_L does not
     }
     if (!have) continue;
-    if (steps == 0 && a.grad_meas) {
-      for (int h = begin; h < track.end; ++h) reinterpret_cast<float2*>(a.grad_meas)[h] = make_float2(0.0f, 0.0f);
-    }
 #pragma unroll
     for (int c = 0; c < 5; ++c) a.grad_seeds[(int64_t)c * N + trk] = b_p[c];
   }

@@ -146,6 +146,12 @@ tpcfit_status from_cuda(cudaError_t e) {
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
+// Zero the gradients of all clusters (null: none wanted): the reverse writes those
+// that a step of a fitted track reaches.
+cudaError_t clear_meas_grad(float* gm, int64_t n_hits, cudaStream_t s) {
+  return gm && n_hits > 0 ? cudaMemsetAsync(gm, 0, 2 * sizeof(float) * (size_t)n_hits, s) : cudaSuccess;
+}
+
 template <class T>
 tpcfit_status grow(T*& ptr, int64_t& cap, int64_t need) {
   if (need <= cap) return TPCFIT_OK;
@@ -589,7 +595,11 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
   if (!h || !hits || n_tracks < 0 || hits->n_hits < 0) return TPCFIT_EINVAL;
   if (!grad_align || !aligned(grad_align, 4)) return TPCFIT_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
-  if (n_tracks == 0) return from_cuda(cudaMemsetAsync(grad_align, 0, sizeof(float) * kAlignFloats, s));
+  if (n_tracks == 0) {
+    cudaError_t e = cudaMemsetAsync(grad_align, 0, sizeof(float) * kAlignFloats, s);
+    if (e == cudaSuccess) e = clear_meas_grad(grad_meas, hits->n_hits, s);
+    return from_cuda(e);
+  }
   if (!track_offsets || !ndf || !grad_chi2 || !grad_seeds) return TPCFIT_EINVAL;
   if (hits->n_hits > 0 && (!hits->y || !hits->z || !hits->rowsec)) return TPCFIT_EINVAL;
   if (!aligned(grad_chi2, 4) || !aligned(grad_seeds, 4) || !aligned(ndf, 4) || (grad_meas && !aligned(grad_meas, 8)))
@@ -645,6 +655,7 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
     b.grad_meas = grad_meas;
     b.grad_align_atomic = grad_align;
     e = cudaMemsetAsync(grad_align, 0, sizeof(float) * kAlignFloats, s);
+    if (e == cudaSuccess) e = clear_meas_grad(grad_meas, hits->n_hits, s);
     if (e == cudaSuccess) e = launch_backward_fast(b, h->bwd_warps, s);
     return from_cuda(e);
   }
@@ -667,7 +678,10 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
   }
   b.grad_meas = gm;
   b.grad_align_atomic = nullptr;
-  e = launch_backward_det(b, h->bwd_warps, s);
+  // the sums below take every cluster, those that no step reaches too (beyond the end
+  // of an outward pass, of no track)
+  e = clear_meas_grad(gm, hits->n_hits, s);
+  if (e == cudaSuccess) e = launch_backward_det(b, h->bwd_warps, s);
   if (h->det_reduce == 0) {
     if (e == cudaSuccess)
       e = launch_key_fixed_reduce(gm, hits->rowsec, hits->n_hits, h->geo.n_rows, h->d_keys, grad_align, s);

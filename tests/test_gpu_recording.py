@@ -124,3 +124,63 @@ def test_offsets_beyond_the_arrays_touch_nothing_outside(kind, where):
                 assert bool(torch.isnan(got[k][~mine]).all()), k
     finally:
         f.close()
+
+
+def _ends_early(n, seed, step=20):
+    """Tracks of which every third has cluster `step` in the sector opposite, where no
+    step leads: its outward pass ends there."""
+    fr = synth.generate(n, seed)
+    fr.rowsec = fr.rowsec.copy()
+    off = fr.offsets.astype(np.int64)
+    early = np.array([t for t in range(0, n, 3) if off[t + 1] - off[t] > step + 5])
+    for t in early:
+        h = off[t] + step
+        row, sec = int(fr.rowsec[h]) >> 6, int(fr.rowsec[h]) & 63
+        fr.rowsec[h] = np.uint16((row << 6) | (sec // 18 * 18 + (sec + 9) % 18))
+    return fr, early, step
+
+
+@pytest.mark.parametrize("reduction", [0, 1])
+@pytest.mark.parametrize("kind", KINDS)
+def test_clusters_that_no_step_reached_have_no_gradient(kind, reduction):
+    # clusters after the end of an outward pass, and clusters of no track at all:
+    # their gradients are zero and no alignment gradient holds what another call,
+    # or nobody, left in their place
+    fr, early, step = _ends_early(300, 63)
+    whole = tf.frame_to_device(fr)
+    dev = dict(whole, offsets=whole["offsets"][1:-1].contiguous(), seeds=whole["seeds"][:, 1:-1].contiguous())
+    off = fr.offsets[1:-1].astype(np.int64)
+    n = 298
+    end = off[1:].copy()
+    inner = early[(early > 0) & (early < 299)]
+    end[inner - 1] = off[inner - 1] + step
+    reached = np.zeros(fr.n_hits, bool)
+    for t in range(n):
+        reached[off[t]:end[t]] = True
+    reached_dev = torch.from_numpy(reached).cuda()
+    g = torch.ones(n, device="cuda")
+    ga = []
+    for used_before in (True, False):
+        f = _fitter(fr, kind)
+        try:
+            f.set_det_reduction(reduction)
+            if used_before:  # the handle's scratch holds large gradients of all clusters
+                straight = tf.frame_to_device(synth.generate(300, 63))
+                out = f.fit(straight)
+                f.backward(straight, out, torch.full((300,), 1e4, device="cuda"))
+            out = f.fit(dev)
+            assert f.status()[0] == tf.OK
+            assert bool((out["ndf"][torch.from_numpy(inner - 1).cuda()] == 2 * step - 5).all())
+            ga.append(f.backward(dev, out, g)[0].reshape(-1, 2).clone())
+            gm = torch.full((fr.n_hits, 2), 9.0, device="cuda")
+            f.backward(dev, out, g, gm)
+            assert bool((gm[~reached_dev] == 0).all()) and bool((gm[reached_dev] != 9.0).all())
+        finally:
+            f.close()
+        # each alignment gradient is minus the sum of its clusters' (FP32 sums of a
+        # few terms: 1e-5 in norm)
+        key = torch.from_numpy((fr.rowsec.astype(np.int64) & 63) * 152 + (fr.rowsec.astype(np.int64) >> 6)).cuda()
+        want = torch.zeros((36 * 152, 2), dtype=torch.float64, device="cuda").index_add_(0, key, -gm.double())
+        assert float((ga[-1].double() - want).norm()) <= 1e-5 * float(want.norm())
+    if KINDS[kind][0]:
+        assert torch.equal(_bits(ga[0]), _bits(ga[1]))
