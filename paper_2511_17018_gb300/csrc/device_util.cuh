@@ -31,6 +31,15 @@ __device__ __forceinline__ int frame_of(const int64_t* base, int n_frames, int64
   return lo;
 }
 
+// A cluster's row and sector by an ordinary load.  Not __ldg: the read-only path is
+// for memory that nobody writes during the launch, and another stream may still be
+// copying a frame in, next to the clusters read or, before its flag, the very ones.
+__device__ __forceinline__ uint16_t load_rowsec(const uint16_t* p) {
+  uint16_t v;
+  asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+  return v;
+}
+
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -695,7 +695,7 @@ __device__ __forceinline__ void stage_window(WarpStage<RPS>& st, const FitArgs& 
       if ((int64_t)h + k >= a.n_hits) break;
       cp_async4(reinterpret_cast<float*>(&st.y[slot][lane]) + k, a.y + h + k);
       cp_async4(reinterpret_cast<float*>(&st.z[slot][lane]) + k, a.z + h + k);
-      reinterpret_cast<uint16_t*>(&st.rs[slot][lane])[k] = __ldg(a.rowsec + h + k);
+      reinterpret_cast<uint16_t*>(&st.rs[slot][lane])[k] = load_rowsec(a.rowsec + h + k);
     }
   }
 }

@@ -185,7 +185,7 @@ __device__ __forceinline__ void stage_issue_lanes(WarpStageLanes<P, RPS>& st, in
       if (wa >= rs_begin && wa + 4 <= rs_end) {
         cp_async4(&st.rs[b][t][k], (const void*)wa);
       } else {
-        st.rs[b][t][k] = (uint32_t)__ldg(rp) << (16u * (unsigned)(((uintptr_t)rp >> 1) & 1u));
+        st.rs[b][t][k] = (uint32_t)load_rowsec(rp) << (16u * (unsigned)(((uintptr_t)rp >> 1) & 1u));
       }
     }
   }
