@@ -30,6 +30,13 @@
  *     that takes a stream only enqueues work on it and returns; argument
  *     errors are returned synchronously before anything is enqueued.
  *   - A handle is not thread-safe; use one handle per host thread.
+ *   - Calls that only launch (the fits, the adjoint, the smoother, the rejection)
+ *     can be captured in a CUDA graph after the same call has run outside the
+ *     capture.  The scratch that a captured call uses stays allocated until
+ *     tpcfit_destroy, also where later calls outgrow it.  A replayed recorded fit
+ *     replaces the recording like the call that was captured: what follows it (the
+ *     adjoint, the smoother) belongs into the same graph, and a recorded fit made
+ *     before the replay is gone.
  */
 #ifndef TPCFIT_H_
 #define TPCFIT_H_

@@ -134,6 +134,10 @@ struct tpcfit_handle {
   int64_t reject_cap = 0;       // ints
   int32_t* d_frame_scratch = nullptr;
   int64_t frame_scratch_cap = 0;
+  // a call was captured: graphs hold the scratch of that time, so what is outgrown
+  // stays until the handle goes
+  bool captured = false;
+  std::vector<void*> outgrown;
 };
 
 namespace {
@@ -152,15 +156,49 @@ cudaError_t clear_meas_grad(float* gm, int64_t n_hits, cudaStream_t s) {
   return gm && n_hits > 0 ? cudaMemsetAsync(gm, 0, 2 * sizeof(float) * (size_t)n_hits, s) : cudaSuccess;
 }
 
-template <class T>
-tpcfit_status grow(T*& ptr, int64_t& cap, int64_t need) {
+// Whether the call's stream is being captured, noted in the handle.
+bool note_capture(tpcfit_handle* h, cudaStream_t s) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &c) != cudaSuccess) {  // the default stream, while others are captured
+    cudaGetLastError();
+    return true;
+  }
+  if (c != cudaStreamCaptureStatusNone) h->captured = true;
+  return c != cudaStreamCaptureStatusNone;
+}
+
+// Let an outgrown buffer go.  A replay of a captured call writes to it all the same,
+// so it is then kept, for the handle's life (without the room to note it, for good).
+void let_go(tpcfit_handle* h, void* p) {
+  if (!p) return;
+  if (!h->captured) {
+    cudaFree(p);
+    return;
+  }
+  try {
+    h->outgrown.push_back(p);
+  } catch (...) {
+  }
+}
+
+// Room for `need` elements of scratch; the contents do not survive.  What a captured
+// handle outgrows stays allocated: there a quarter more is taken, so that all the
+// outgrown buffers together are at most four times the last one.
+template <class T, class C>
+tpcfit_status grow(tpcfit_handle* h, T*& ptr, C& cap, C need) {
   if (need <= cap) return TPCFIT_OK;
-  if (ptr) cudaFree(ptr);
+  let_go(h, ptr);
   ptr = nullptr;
   cap = 0;
-  cudaError_t e = cudaMalloc(&ptr, sizeof(T) * (size_t)need);
+  C take = h->captured ? need + need / 4 : need;
+  cudaError_t e = cudaMalloc(&ptr, sizeof(T) * (size_t)take);
+  if (e == cudaErrorMemoryAllocation && take > need) {
+    cudaGetLastError();
+    take = need;
+    e = cudaMalloc(&ptr, sizeof(T) * (size_t)take);
+  }
   if (e != cudaSuccess) return from_cuda(e);
-  cap = need;
+  cap = take;
   return TPCFIT_OK;
 }
 
@@ -180,7 +218,7 @@ tpcfit_status ensure_pipe(tpcfit_handle* h) {
 // Room for the tape of a recorded fit (kernel_abi.h) and its shape; without one
 // (a.tape null) the fit leaves checkpoints: another form of fit, no memory, or a
 // tape of more than half of what is free.
-void ensure_tape(tpcfit_handle* h, FitArgs& a, cudaStream_t s) {
+void ensure_tape(tpcfit_handle* h, FitArgs& a, bool capturing) {
   const bool ud = a.form == 1;
   if (h->lanes_per_track != 1 || !(h->deterministic || a.mat || ud)) return;
   const int64_t T = item_tracks(a.n_tracks, h->sms);
@@ -197,24 +235,22 @@ void ensure_tape(tpcfit_handle* h, FitArgs& a, cudaStream_t s) {
                                          : items * tape_rows(ud, kMaxRows, every);
   if (rows > INT32_MAX) return;
   const int64_t need = rows * T;
-  if (need > h->tape_cap || items > h->tape_item_cap) {
-    // nothing is allocated while the stream is being captured
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return;
-  }
+  // nothing is allocated while the stream is being captured
+  if (capturing && (need > h->tape_cap || items > h->tape_item_cap)) return;
   if (need > h->tape_cap) {
     size_t avail = 0, total = 0;
     if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
       cudaGetLastError();
       return;
     }
-    if (sizeof(float4) * (uint64_t)need > (avail + sizeof(float4) * (uint64_t)h->tape_cap) / 2) return;
-    if (grow(h->d_tape, h->tape_cap, need) != TPCFIT_OK) {
+    const int64_t given_back = h->captured ? 0 : h->tape_cap;
+    if (sizeof(float4) * (uint64_t)need > (avail + sizeof(float4) * (uint64_t)given_back) / 2) return;
+    if (grow(h, h->d_tape, h->tape_cap, need) != TPCFIT_OK) {
       cudaGetLastError();
       return;
     }
   }
-  if (grow(h->d_tape_item, h->tape_item_cap, items) != TPCFIT_OK) {
+  if (grow(h, h->d_tape_item, h->tape_item_cap, items) != TPCFIT_OK) {
     cudaGetLastError();
     return;
   }
@@ -239,7 +275,7 @@ tpcfit_status ensure_perm(tpcfit_handle* h, int64_t n) {
       cudaFree(p);
       return from_cuda(e);
     }
-    cudaFree(h->d_perm);
+    let_go(h, h->d_perm);
   }
   h->d_perm = p;
   h->perm_cap = n;
@@ -332,6 +368,7 @@ void tpcfit_destroy(tpcfit_handle* h) {
   if (h->d_keys) cudaFree(h->d_keys);
   if (h->d_frame_scratch) cudaFree(h->d_frame_scratch);
   if (h->d_reject) cudaFree(h->d_reject);
+  for (void* p : h->outgrown) cudaFree(p);
   delete h;
 }
 
@@ -379,6 +416,7 @@ tpcfit_status tpcfit_fit(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
     return TPCFIT_EINVAL;
   if (hits->n_hits > INT32_MAX) return TPCFIT_EINVAL;  // int32 track offsets
   cudaStream_t s = (cudaStream_t)stream;
+  const bool capturing = note_capture(h, s);
   tpcfit_status st = TPCFIT_OK;
   FitArgs a{};
   a.geo = h->geo;
@@ -403,14 +441,14 @@ tpcfit_status tpcfit_fit(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
   h->rec_valid = false;
   if (h->record) {
     const int64_t slots = hits->n_hits / kCkptEvery + (int64_t)n_tracks + 1;
-    st = grow(h->d_ck, h->ck_cap, 2 * slots * kCkptFloats);
-    if (st == TPCFIT_OK) st = grow(h->d_ck_last, h->ck_last_cap, (int64_t)n_tracks);
+    st = grow(h, h->d_ck, h->ck_cap, 2 * slots * kCkptFloats);
+    if (st == TPCFIT_OK) st = grow(h, h->d_ck_last, h->ck_last_cap, (int64_t)n_tracks);
     if (st != TPCFIT_OK) return st;
     a.ck = h->d_ck;
     a.ck_last = h->d_ck_last;
     a.ck_slots = slots;
     h->ck_slots = slots;
-    ensure_tape(h, a, s);
+    ensure_tape(h, a, capturing);
     h->rec_sorted = h->sort_by_length != 0;
     h->rec_tape = a.tape != nullptr;
     h->rec_every = a.tape_every;
@@ -454,8 +492,9 @@ tpcfit_status tpcfit_fit_frames(tpcfit_handle* h, const tpcfit_hits* hits, const
   // ready flags are set by work on other streams; on the legacy default stream
   // that work would wait for the fit itself
   if (frame_ready && (s == nullptr || s == cudaStreamLegacy)) return TPCFIT_EINVAL;
+  note_capture(h, s);
   tpcfit_status st = ensure_perm(h, n_tracks);
-  if (st == TPCFIT_OK) st = grow(h->d_frame_scratch, h->frame_scratch_cap, frame_order_scratch_ints(n_frames));
+  if (st == TPCFIT_OK) st = grow(h, h->d_frame_scratch, h->frame_scratch_cap, frame_order_scratch_ints(n_frames));
   if (st != TPCFIT_OK) return st;
   FitArgs a{};
   a.geo = h->geo;
@@ -505,7 +544,8 @@ tpcfit_status tpcfit_reject_outliers(tpcfit_handle* h, const tpcfit_hits* hits, 
     if (!hits->y || !hits->z || !hits->rowsec || !chi2 || !y_out || !z_out || !rowsec_out) return TPCFIT_EINVAL;
     if (!aligned(chi2, 4) || !aligned(y_out, 4) || !aligned(z_out, 4) || !aligned(rowsec_out, 2)) return TPCFIT_EINVAL;
   }
-  tpcfit_status st = grow(h->d_reject, h->reject_cap, reject_scratch_ints(n_tracks));
+  note_capture(h, (cudaStream_t)stream);
+  tpcfit_status st = grow(h, h->d_reject, h->reject_cap, reject_scratch_ints(n_tracks));
   if (st != TPCFIT_OK) return st;
   return from_cuda(launch_reject(track_offsets, n_tracks, hits->y, hits->z, hits->rowsec, hits->n_hits, chi2,
                                  chi2_cut, y_out, z_out, rowsec_out, offsets_out, h->d_reject,
@@ -607,6 +647,7 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
   if (!h->rec_valid || h->rec_tracks != n_tracks || h->rec_hits != hits->n_hits ||
       h->rec_det != h->deterministic)
     return TPCFIT_ESTATE;
+  note_capture(h, s);
   tpcfit_status st = TPCFIT_OK;
   BwdArgs b{};
   b.geo = h->geo;
@@ -647,7 +688,7 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
   e = h->deterministic ? backward_store_det(h->bwd_warps, b.phys, b.form, need)
                        : backward_store_fast(h->bwd_warps, b.phys, b.form, need);
   if (e != cudaSuccess) return from_cuda(e);
-  st = grow(h->d_seg, h->seg_cap, need);
+  st = grow(h, h->d_seg, h->seg_cap, need);
   if (st != TPCFIT_OK) return st;
   b.seg = h->d_seg;
   if (!h->deterministic) {
@@ -663,19 +704,13 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
   // fixed-order sums per key
   float* gm = grad_meas;
   if (!gm) {
-    st = grow(h->d_gm, h->gm_cap, 2 * hits->n_hits);
+    st = grow(h, h->d_gm, h->gm_cap, 2 * hits->n_hits);
     if (st != TPCFIT_OK) return st;
     gm = h->d_gm;
   }
   const size_t kb = h->det_reduce == 1 ? key_sort_scratch_bytes(hits->n_hits) : key_fixed_scratch_bytes();
-  if (kb > h->keys_cap) {
-    if (h->d_keys) cudaFree(h->d_keys);
-    h->d_keys = nullptr;
-    h->keys_cap = 0;
-    e = cudaMalloc(&h->d_keys, kb);
-    if (e != cudaSuccess) return from_cuda(e);
-    h->keys_cap = kb;
-  }
+  st = grow(h, h->d_keys, h->keys_cap, kb);
+  if (st != TPCFIT_OK) return st;
   b.grad_meas = gm;
   b.grad_align_atomic = nullptr;
   // the sums below take every cluster, those that no step reaches too (beyond the end
@@ -711,6 +746,7 @@ tpcfit_status run_smooth(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
       h->rec_det != h->deterministic)
     return TPCFIT_ESTATE;
   cudaStream_t s = (cudaStream_t)stream;
+  note_capture(h, s);
   tpcfit_status st = TPCFIT_OK;
   SmoothArgs a{};
   a.geo = h->geo;
@@ -742,7 +778,7 @@ tpcfit_status run_smooth(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
   int64_t need = 0;
   cudaError_t e = h->deterministic ? smooth_store_det(need) : smooth_store_fast(need);
   if (e != cudaSuccess) return from_cuda(e);
-  st = grow(h->d_seg, h->seg_cap, need);
+  st = grow(h, h->d_seg, h->seg_cap, need);
   if (st != TPCFIT_OK) return st;
   a.seg = h->d_seg;
   e = h->deterministic ? launch_smooth_det(a, s) : launch_smooth_fast(a, s);

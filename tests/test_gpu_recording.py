@@ -184,3 +184,42 @@ def test_clusters_that_no_step_reached_have_no_gradient(kind, reduction):
         assert float((ga[-1].double() - want).norm()) <= 1e-5 * float(want.norm())
     if KINDS[kind][0]:
         assert torch.equal(_bits(ga[0]), _bits(ga[1]))
+
+
+def test_a_captured_fit_and_adjoint_outlive_larger_calls():
+    # the graph's tape and scratch stay in place while the handle goes on to fits
+    # that need more of both
+    fr = synth.generate(3000, 65, drop_p=0.05, cap_lengths=True)
+    dev = tf.frame_to_device(fr)
+    large = tf.frame_to_device(synth.generate(20000, 66))
+    g, g_large = torch.ones(3000, device="cuda"), torch.ones(20000, device="cuda")
+    f = tf.Fitter(fr.geometry, fr.bz)
+    try:
+        f.set_record(True)
+        out = tf.empty_outputs(3000)
+        ga, gs = f.backward(dev, f.fit(dev, out), g)
+        want = {k: out[k].clone() for k in out}
+        ga0, gs0 = ga.clone(), gs.clone()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            ga, gs = f.backward(dev, f.fit(dev, out), g)
+        for det in (True, False):
+            f.set_mode(det)
+            o = f.fit(large)
+            f.backward(large, o, g_large)
+            f.smooth(large, o)
+        junk = [torch.full((1 << 26,), 3.0, device="cuda") for _ in range(8)]  # takes what was given back
+        torch.cuda.synchronize()
+        for t in (*out.values(), gs):
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        for k in out:
+            assert torch.equal(_bits(out[k]), _bits(want[k])), k
+        assert torch.equal(_bits(gs), _bits(gs0))
+        assert float((ga - ga0).norm()) <= 1e-5 * float(ga0.norm())
+        assert all(bool((t == 3.0).all()) for t in junk)
+        del graph
+    finally:
+        f.close()
