@@ -181,6 +181,18 @@ void let_go(tpcfit_handle* h, void* p) {
   }
 }
 
+// Scratch of `n` elements.  A refused allocation is the call's own answer (ENOMEM): it
+// is not left behind for the next launch to report.
+template <class T>
+cudaError_t alloc(T*& p, size_t n) {
+  const cudaError_t e = cudaMalloc(&p, sizeof(T) * n);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+  }
+  return e;
+}
+
 // Room for `need` elements of scratch; the contents do not survive.  What a captured
 // handle outgrows stays allocated: there a quarter more is taken, so that all the
 // outgrown buffers together are at most four times the last one.
@@ -191,11 +203,10 @@ tpcfit_status grow(tpcfit_handle* h, T*& ptr, C& cap, C need) {
   ptr = nullptr;
   cap = 0;
   C take = h->captured ? need + need / 4 : need;
-  cudaError_t e = cudaMalloc(&ptr, sizeof(T) * (size_t)take);
+  cudaError_t e = alloc(ptr, (size_t)take);
   if (e == cudaErrorMemoryAllocation && take > need) {
-    cudaGetLastError();
     take = need;
-    e = cudaMalloc(&ptr, sizeof(T) * (size_t)take);
+    e = alloc(ptr, (size_t)take);
   }
   if (e != cudaSuccess) return from_cuda(e);
   cap = take;
@@ -245,15 +256,9 @@ void ensure_tape(tpcfit_handle* h, FitArgs& a, bool capturing) {
     }
     const int64_t given_back = h->captured ? 0 : h->tape_cap;
     if (sizeof(float4) * (uint64_t)need > (avail + sizeof(float4) * (uint64_t)given_back) / 2) return;
-    if (grow(h, h->d_tape, h->tape_cap, need) != TPCFIT_OK) {
-      cudaGetLastError();
-      return;
-    }
+    if (grow(h, h->d_tape, h->tape_cap, need) != TPCFIT_OK) return;
   }
-  if (grow(h, h->d_tape_item, h->tape_item_cap, items) != TPCFIT_OK) {
-    cudaGetLastError();
-    return;
-  }
+  if (grow(h, h->d_tape_item, h->tape_item_cap, items) != TPCFIT_OK) return;
   a.tape = h->d_tape;
   a.tape_item = h->d_tape_item;
   a.tape_rows = rows;
@@ -265,7 +270,7 @@ void ensure_tape(tpcfit_handle* h, FitArgs& a, bool capturing) {
 tpcfit_status ensure_perm(tpcfit_handle* h, int64_t n) {
   if (n <= h->perm_cap) return TPCFIT_OK;
   int32_t* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, sizeof(int32_t) * (size_t)n);
+  cudaError_t e = alloc(p, (size_t)n);
   if (e != cudaSuccess) return from_cuda(e);
   if (h->d_perm) {
     e = cudaDeviceSynchronize();
@@ -327,10 +332,10 @@ tpcfit_status tpcfit_create(const tpcfit_geometry* geometry, double bz_tesla, tp
   }
   cudaError_t e = cudaGetDevice(&h->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_align, sizeof(float) * kAlignFloats);
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_err, sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_work, sizeof(unsigned int) * 64);
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_sort_scratch, sizeof(int32_t) * 512);
+  if (e == cudaSuccess) e = alloc(h->d_align, kAlignFloats);
+  if (e == cudaSuccess) e = alloc(h->d_err, 1);
+  if (e == cudaSuccess) e = alloc(h->d_work, 64);
+  if (e == cudaSuccess) e = alloc(h->d_sort_scratch, 512);
   if (e == cudaSuccess) e = cudaMemset(h->d_align, 0, sizeof(float) * kAlignFloats);
   if (e == cudaSuccess) e = cudaMemset(h->d_err, 0, sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -820,7 +825,7 @@ tpcfit_status tpcfit_fit_host(tpcfit_handle* h, const float* y, const float* z, 
     if (h->d_stage) cudaFree(h->d_stage);
     h->d_stage = nullptr;
     h->stage_cap = 0;
-    e = cudaMalloc(&h->d_stage, total);
+    e = alloc(h->d_stage, total);
     if (e != cudaSuccess) return from_cuda(e);
     h->stage_cap = total;
   }
@@ -913,7 +918,7 @@ tpcfit_status tpcfit_fit_adjoint_host(tpcfit_handle* h, const float* y, const fl
     if (h->d_pipe[slot]) cudaFree(h->d_pipe[slot]);
     h->d_pipe[slot] = nullptr;
     h->pipe_cap[slot] = 0;
-    e = cudaMalloc(&h->d_pipe[slot], total);
+    e = alloc(h->d_pipe[slot], total);
     if (e != cudaSuccess) return from_cuda(e);
     h->pipe_cap[slot] = total;
   }

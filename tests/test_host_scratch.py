@@ -122,3 +122,15 @@ def test_a_captured_handle_that_keeps_growing_stays_bounded(lib):
     # a quarter more each time: the last one at most 1.25 times the need, those before
     # it together at most four times the last
     assert total[1] <= 5 * 1.25 * total[0]
+
+
+def test_a_refused_allocation_leaves_nothing_behind(lib):
+    # ENOMEM is that call's answer; the next call, which fits, does not report it
+    h = Handle(lib, limit=GB)
+    try:
+        assert h.fit(10_000_000, per=200) == 3
+        assert h.fit(5000) == 0 and h.backward(5000) == 0
+        assert lib.tpcfit_reserve(h.h, C.c_int64(2_000_000_000), C.c_int64(0)) == 3
+        assert h.fit(5000) == 0
+    finally:
+        h.close()
