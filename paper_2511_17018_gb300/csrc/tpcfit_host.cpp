@@ -193,6 +193,22 @@ cudaError_t alloc(T*& p, size_t n) {
   return e;
 }
 
+// The same for the fits and what stages their inputs: where there is no room, the tape
+// gives way, which the fit can do without (it then leaves checkpoints) and which no
+// recording needs any more.
+template <class T>
+cudaError_t alloc_or_take_tape(tpcfit_handle* h, T*& p, size_t n) {
+  cudaError_t e = alloc(p, n);
+  if (e == cudaErrorMemoryAllocation && h->d_tape && !h->captured) {
+    h->rec_valid = false;
+    cudaFree(h->d_tape);
+    h->d_tape = nullptr;
+    h->tape_cap = 0;
+    e = alloc(p, n);
+  }
+  return e;
+}
+
 // Room for `need` elements of scratch; the contents do not survive.  What a captured
 // handle outgrows stays allocated: there a quarter more is taken, so that all the
 // outgrown buffers together are at most four times the last one.
@@ -208,6 +224,7 @@ tpcfit_status grow(tpcfit_handle* h, T*& ptr, C& cap, C need) {
     take = need;
     e = alloc(ptr, (size_t)take);
   }
+  if (e == cudaErrorMemoryAllocation && !h->rec_valid) e = alloc_or_take_tape(h, ptr, (size_t)take);
   if (e != cudaSuccess) return from_cuda(e);
   cap = take;
   return TPCFIT_OK;
@@ -248,6 +265,7 @@ void ensure_tape(tpcfit_handle* h, FitArgs& a, bool capturing) {
   const int64_t need = rows * T;
   // nothing is allocated while the stream is being captured
   if (capturing && (need > h->tape_cap || items > h->tape_item_cap)) return;
+  if (grow(h, h->d_tape_item, h->tape_item_cap, items) != TPCFIT_OK) return;
   if (need > h->tape_cap) {
     size_t avail = 0, total = 0;
     if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
@@ -258,7 +276,6 @@ void ensure_tape(tpcfit_handle* h, FitArgs& a, bool capturing) {
     if (sizeof(float4) * (uint64_t)need > (avail + sizeof(float4) * (uint64_t)given_back) / 2) return;
     if (grow(h, h->d_tape, h->tape_cap, need) != TPCFIT_OK) return;
   }
-  if (grow(h, h->d_tape_item, h->tape_item_cap, items) != TPCFIT_OK) return;
   a.tape = h->d_tape;
   a.tape_item = h->d_tape_item;
   a.tape_rows = rows;
@@ -270,7 +287,7 @@ void ensure_tape(tpcfit_handle* h, FitArgs& a, bool capturing) {
 tpcfit_status ensure_perm(tpcfit_handle* h, int64_t n) {
   if (n <= h->perm_cap) return TPCFIT_OK;
   int32_t* p = nullptr;
-  cudaError_t e = alloc(p, (size_t)n);
+  cudaError_t e = h->rec_valid ? alloc(p, (size_t)n) : alloc_or_take_tape(h, p, (size_t)n);
   if (e != cudaSuccess) return from_cuda(e);
   if (h->d_perm) {
     e = cudaDeviceSynchronize();
@@ -444,6 +461,10 @@ tpcfit_status tpcfit_fit(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
   a.mat = h->geo.mat;
   a.field = h->geo.field;
   h->rec_valid = false;
+  if (h->sort_by_length) {  // (before the tape, which would give way to it)
+    st = ensure_perm(h, n_tracks);
+    if (st != TPCFIT_OK) return st;
+  }
   if (h->record) {
     const int64_t slots = hits->n_hits / kCkptEvery + (int64_t)n_tracks + 1;
     st = grow(h, h->d_ck, h->ck_cap, 2 * slots * kCkptFloats);
@@ -459,8 +480,6 @@ tpcfit_status tpcfit_fit(tpcfit_handle* h, const tpcfit_hits* hits, const int32_
     h->rec_every = a.tape_every;
   }
   if (h->sort_by_length) {
-    st = ensure_perm(h, n_tracks);
-    if (st != TPCFIT_OK) return st;
     cudaError_t e = launch_length_order(track_offsets, n_tracks, h->d_perm, h->d_sort_scratch, s);
     if (e != cudaSuccess) return from_cuda(e);
     a.perm = h->d_perm;
@@ -498,6 +517,7 @@ tpcfit_status tpcfit_fit_frames(tpcfit_handle* h, const tpcfit_hits* hits, const
   // that work would wait for the fit itself
   if (frame_ready && (s == nullptr || s == cudaStreamLegacy)) return TPCFIT_EINVAL;
   note_capture(h, s);
+  h->rec_valid = false;  // the adjoint follows single-frame fits only
   tpcfit_status st = ensure_perm(h, n_tracks);
   if (st == TPCFIT_OK) st = grow(h, h->d_frame_scratch, h->frame_scratch_cap, frame_order_scratch_ints(n_frames));
   if (st != TPCFIT_OK) return st;
@@ -526,7 +546,6 @@ tpcfit_status tpcfit_fit_frames(tpcfit_handle* h, const tpcfit_hits* hits, const
   a.frame_align = frame_alignment;
   a.frame_ready = frame_ready;
   a.wait_ns = wait_timeout_ns > 0 ? wait_timeout_ns : 1000000000LL;
-  h->rec_valid = false;  // the adjoint follows single-frame fits only
   cudaError_t e =
       launch_frame_length_order(track_offsets, n_tracks, frame_track_base, n_frames, h->d_perm, h->d_frame_scratch, s);
   if (e != cudaSuccess) return from_cuda(e);
@@ -825,7 +844,7 @@ tpcfit_status tpcfit_fit_host(tpcfit_handle* h, const float* y, const float* z, 
     if (h->d_stage) cudaFree(h->d_stage);
     h->d_stage = nullptr;
     h->stage_cap = 0;
-    e = alloc(h->d_stage, total);
+    e = alloc_or_take_tape(h, h->d_stage, total);
     if (e != cudaSuccess) return from_cuda(e);
     h->stage_cap = total;
   }
@@ -918,7 +937,7 @@ tpcfit_status tpcfit_fit_adjoint_host(tpcfit_handle* h, const float* y, const fl
     if (h->d_pipe[slot]) cudaFree(h->d_pipe[slot]);
     h->d_pipe[slot] = nullptr;
     h->pipe_cap[slot] = 0;
-    e = alloc(h->d_pipe[slot], total);
+    e = alloc_or_take_tape(h, h->d_pipe[slot], total);
     if (e != cudaSuccess) return from_cuda(e);
     h->pipe_cap[slot] = total;
   }

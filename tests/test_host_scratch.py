@@ -134,3 +134,32 @@ def test_a_refused_allocation_leaves_nothing_behind(lib):
         assert h.fit(5000) == 0
     finally:
         h.close()
+
+
+def test_the_tape_gives_way_to_what_a_fit_cannot_do_without(lib):
+    # 4.6 GB: a recorded fit of 200,000 tracks takes 1.9 GB for its tape; checkpoints of
+    # 1.6 million tracks (3.0 GB) fit without it, in a handle that never had one too
+    limit = 4600 << 20
+    for first in (False, True):
+        h = Handle(lib, limit)
+        try:
+            if first:
+                assert h.fit(200_000) == 0 and lib.fake_taped()
+                assert h.backward(200_000) == 0
+            lib.fake_forget()
+            assert h.fit(1_600_000) == 0 and not lib.fake_taped()
+            assert h.backward(1_600_000) == 0
+            assert lib.fake_used_live() == lib.fake_used()
+        finally:
+            h.close()
+
+
+def test_the_tape_stays_while_its_recording_does(lib):
+    # scratch of other calls that finds no room is refused; the recording goes on
+    h = Handle(lib, 2500 << 20)
+    try:
+        assert h.fit(100_000) == 0 and lib.fake_taped()
+        assert lib.tpcfit_reserve(h.h, C.c_int64(1_000_000_000), C.c_int64(0)) == 3
+        assert h.backward(100_000) == 0 and h.smooth(100_000) == 0
+    finally:
+        h.close()
