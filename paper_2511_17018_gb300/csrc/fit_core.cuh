@@ -657,10 +657,12 @@ struct TrackState {
 // each group of lanes taking consecutive ones of one track, cost about 38 of the
 // step's 340 instructions: shuffles, bounds of the rowsec words, three copies and
 // their addresses per cluster.)  y and z bypass L1, whose room the alignment tables
-// need.  A window that reaches beyond the arrays, or any window where the arrays
-// are not aligned, is copied cluster by cluster.  Plain fit of 400,000 tracks: 725
-// -> 657 us (666 through L1; 699 through L1 with a ring of 4 windows, whose shared
-// memory comes out of L1), recorded 980 -> 897.
+// need.  Plain fit of 400,000 tracks: 725 -> 657 us (666 through L1; 699 through L1
+// with a ring of 4 windows, whose shared memory comes out of L1), recorded 980 -> 897.
+// Arrays that begin within a window, all three at the same place, are staged in
+// windows just the same (400,000 tracks, arrays one element after an aligned address:
+// 665 us; cluster by cluster 1,250, with the copies of single clusters 740).  A window
+// that reaches beyond the arrays is copied cluster by cluster.
 template <int RPS>
 struct WarpStage {
   static constexpr int kWindows = fit_stage_windows(RPS);
@@ -669,29 +671,59 @@ struct WarpStage {
   uint2 rs[kWindows][kWarp];
 };
 
-// The windows of one lane's pass: step i is hit first + dir i, window r is
-// (first >> 2) + dir r, and `last` the largest r that holds a step.
+// The windows of one lane's pass, in hits shifted by win_shift: step i is hit
+// first + dir i, window r is (first >> 2) + dir r, and `last` the largest r that holds
+// a step.
 struct LaneWindows {
   int base, dir, last;
 };
 
-__device__ __forceinline__ bool windows_aligned(const FitArgs& a) {
-  return (((uintptr_t)a.y | (uintptr_t)a.z) & 15u) == 0 && ((uintptr_t)a.rowsec & 7u) == 0;
+// A window inside the arrays, aligned in y, whose z and rowsec are not: they are copied
+// in the largest pieces that their alignment allows.  (Source and destination of a
+// piece are both aligned to its size: the destinations begin at 16 and 8 bytes.)
+__device__ __forceinline__ void stage_mixed(float4* z, uint2* rs, const float* zs, const uint16_t* rss) {
+  if (((uintptr_t)zs & 15u) == 0) {
+    cp_async16(z, zs);
+  } else if (((uintptr_t)zs & 7u) == 0) {
+    cp_async8(z, zs);
+    cp_async8(&z->z, zs + 2);
+  } else {
+    cp_async4(&z->x, zs);
+    cp_async4(&z->y, zs + 1);
+    cp_async4(&z->z, zs + 2);
+    cp_async4(&z->w, zs + 3);
+  }
+  if (((uintptr_t)rss & 7u) == 0) {
+    cp_async8(rs, rss);
+  } else if (((uintptr_t)rss & 3u) == 0) {
+    cp_async4(rs, rss);
+    cp_async4(&rs->y, rss + 2);
+  } else {
+    const unsigned v0 = load_rowsec(rss), v1 = load_rowsec(rss + 1), v2 = load_rowsec(rss + 2), v3 = load_rowsec(rss + 3);
+    *rs = make_uint2(v0 | (v1 << 16), v2 | (v3 << 16));
+  }
 }
 
-template <int RPS>
+// MIXED: for arrays that do not share their windows (set_windows in internal.h).
+// SHIFTED: for arrays that begin within a window.
+template <int RPS, bool MIXED, bool SHIFTED>
 __device__ __forceinline__ void stage_window(WarpStage<RPS>& st, const FitArgs& a, const LaneWindows& L, int r,
-                                             bool aligned, int lane) {
+                                             int lane) {
   if (r > L.last) return;
   const int slot = (unsigned)r % (unsigned)WarpStage<RPS>::kWindows;
-  const int h = (L.base + L.dir * r) * 4;
-  if (aligned && (int64_t)h + 4 <= a.n_hits) {
+  const int h = (L.base + L.dir * r) * 4 - (SHIFTED ? a.win_shift : 0);
+  if (__builtin_expect((unsigned)h < a.win_whole, 1)) {
     cp_async16(&st.y[slot][lane], a.y + h);
-    cp_async16(&st.z[slot][lane], a.z + h);
-    cp_async8(&st.rs[slot][lane], a.rowsec + h);
+    if (MIXED) {
+      stage_mixed(&st.z[slot][lane], &st.rs[slot][lane], a.z + h, a.rowsec + h);
+    } else {
+      cp_async16(&st.z[slot][lane], a.z + h);
+      cp_async8(&st.rs[slot][lane], a.rowsec + h);
+    }
   } else {
 #pragma unroll 1
     for (int k = 0; k < 4; ++k) {
+      if (SHIFTED && h + k < 0) continue;
       if ((int64_t)h + k >= a.n_hits) break;
       cp_async4(reinterpret_cast<float*>(&st.y[slot][lane]) + k, a.y + h + k);
       cp_async4(reinterpret_cast<float*>(&st.z[slot][lane]) + k, a.z + h + k);
@@ -795,10 +827,12 @@ __device__ __forceinline__ void write_tape(float4* dst, int pitch, const TrackSt
 // the square-root factor with Potter's updates (the canonical sequence of the
 // deterministic mode), 1 U-D with Bierman's (fast mode, no material layers).
 // RECORD: 0 nothing, 1 checkpoints, 2 the tape.
-template <int RPS, int WARPS, int MINB, int RECORD, bool FRAMES, int PHYS, int FORM = 0>
+// MIXED: the arrays do not share their windows.
+template <int RPS, int WARPS, int MINB, int RECORD, bool FRAMES, int PHYS, int FORM = 0, bool MIXED = false>
 __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_constant__ FitArgs a) {
   const GeoRef& G = TPCFIT_GEO(a);
   constexpr bool MAT = (PHYS & 1) != 0;
+  constexpr bool kShifted = fit_shifted(RPS, WARPS, MINB);
   constexpr int FIELD = (PHYS & 2) ? 1 : 0;
   static_assert(FORM == 0 || (!MAT && !TPCFIT_DET), "the U-D fit: fast mode without material layers");
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -812,7 +846,6 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
   const float* const y_ring = reinterpret_cast<const float*>(&st.y[0][lane]);  // this lane's
   const float* const z_ring = reinterpret_cast<const float*>(&st.z[0][lane]);
   const uint16_t* const rs_ring = reinterpret_cast<const uint16_t*>(&st.rs[0][lane]);
-  const bool aligned = windows_aligned(a);
   const int64_t n_items = ((int64_t)a.n_tracks + a.item_tracks - 1) / a.item_tracks;
 
 #pragma unroll 1
@@ -908,24 +941,25 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
       if (count_max == 0) continue;
       constexpr int kRefill = RPS / 4;  // windows
       LaneWindows L;
-      L.base = my_first >> 2;
+      const int first_at = my_first + (kShifted ? a.win_shift : 0);
+      L.base = first_at >> 2;
       L.dir = dir;
-      L.last = my_count > 0 ? dir * (((my_first + dir * (my_count - 1)) >> 2) - L.base) : -1;
+      L.last = my_count > 0 ? dir * (((first_at + dir * (my_count - 1)) >> 2) - L.base) : -1;
 #pragma unroll
-      for (int r = 0; r <= kRefill; ++r) stage_window<RPS>(st, a, L, r, aligned, lane);
+      for (int r = 0; r <= kRefill; ++r) stage_window<RPS, MIXED, kShifted>(st, a, L, r, lane);
       cp_async_commit();
 #pragma unroll 1
       for (int c0 = 0; c0 < count_max; c0 += RPS) {
         // the windows of the refill after this one
 #pragma unroll
-        for (int r = 1; r <= kRefill; ++r) stage_window<RPS>(st, a, L, c0 / 4 + kRefill + r, aligned, lane);
+        for (int r = 1; r <= kRefill; ++r) stage_window<RPS, MIXED, kShifted>(st, a, L, c0 / 4 + kRefill + r, lane);
         cp_async_commit();
         cp_async_wait<1>();
 #pragma unroll 1
         for (int k = 0; k < RPS; ++k) {
           const int i = c0 + k;
           if (!go || i >= my_count) continue;
-          const int h = my_first + dir * i;
+          const int h = first_at + dir * i;
           const unsigned slot = (unsigned)(dir * ((h >> 2) - L.base)) % (unsigned)WarpStage<RPS>::kWindows;
           // the cluster's place, the same in all three rings (1,000 tracks: 166 -> 158
           // us; an address each had the lane number read anew every step)
@@ -1064,11 +1098,11 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) fit_kernel(const __grid_cons
 }
 
 #ifndef __CUDACC_RTC__
-template <int RPS, int WARPS, int MINB, int RECORD, bool FRAMES, int PHYS, int FORM>
+template <int RPS, int WARPS, int MINB, int RECORD, bool FRAMES, int PHYS, int FORM, bool MIXED = false>
 cudaError_t launch_cfg(const FitArgs& a, cudaStream_t s) {
   constexpr int kThreads = WARPS * 32;
   const size_t smem = sizeof(BlockSmem) + WARPS * sizeof(WarpStage<RPS>);
-  auto kernel = fit_kernel<RPS, WARPS, MINB, RECORD, FRAMES, PHYS, FORM>;
+  auto kernel = fit_kernel<RPS, WARPS, MINB, RECORD, FRAMES, PHYS, FORM, MIXED>;
   static Resident r;
   cudaError_t e = resident_blocks(kernel, kThreads, smem, r);
   if (e != cudaSuccess) return e;
@@ -1076,6 +1110,7 @@ cudaError_t launch_cfg(const FitArgs& a, cudaStream_t s) {
   const WorkShape w = work_shape(a.n_tracks, r.blocks < most ? r.blocks : most, WARPS, r.sms);
   FitArgs b = a;
   b.item_tracks = w.tracks;
+  set_windows(b, MIXED, fit_shifted(RPS, WARPS, MINB));
   e = clear_work(a.work, RECORD == 2, needs_work_counter(w), s);
   if (e != cudaSuccess) return e;
   kernel<<<w.blocks, w.warps * kWarp, sizeof(BlockSmem) + w.warps * sizeof(WarpStage<RPS>), s>>>(b);
@@ -1103,6 +1138,12 @@ cudaError_t launch_default(const FitArgs& a, cudaStream_t s) {
     if (warps <= 8) return launch_cfg<4, 8, 1, RECORD, FRAMES, PHYS, FORM>(a, s);
     if (warps <= 16) return launch_cfg<4, 16, 1, RECORD, FRAMES, PHYS, FORM>(a, s);
   }
+  // arrays without common windows: cluster by cluster, a full batch's staging takes
+  // longer than its arithmetic (400,000 tracks: 1,190 to 1,250 us against 665 aligned,
+  // 700 to 740 so); smaller batches wait for their tracks' chains either way.  (The fast
+  // square-root form keeps one kernel: see above.)
+  if constexpr (RECORD != 1 && (TPCFIT_DET || FORM == 1))
+    if (mixed_windows(a)) return launch_cfg<4, 24, 1, RECORD, FRAMES, PHYS, FORM, true>(a, s);
   return launch_cfg<4, 24, 1, RECORD, FRAMES, PHYS, FORM>(a, s);
 }
 

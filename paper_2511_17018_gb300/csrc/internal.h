@@ -72,6 +72,24 @@ inline WorkShape work_shape(int64_t n_tracks, int resident, int max_warps, int s
 }
 inline bool needs_work_counter(const WorkShape& w) { return w.items > w.blocks * w.warps; }
 
+// The windows in which the fit stages clusters (WarpStage in fit_core.cuh): four
+// clusters that are aligned in y, wherever in a window the array begins.  Arrays taken
+// from larger ones at one offset begin at the same place, so that z and rowsec share
+// the windows; where they do not (mixed), only a kernel made for it copies windows.
+// mixed_kernel, shifted: what the kernel is made for; it copies cluster by cluster what
+// it is not made for.
+inline int window_place(const void* p, size_t element) { return (int)((uintptr_t)p / element) & 3; }
+inline bool mixed_windows(const FitArgs& a) {
+  const int y = window_place(a.y, sizeof(float));
+  return y != window_place(a.z, sizeof(float)) || y != window_place(a.rowsec, sizeof(uint16_t));
+}
+inline void set_windows(FitArgs& a, bool mixed_kernel, bool shifted) {
+  const int place = window_place(a.y, sizeof(float));
+  const bool fits = a.n_hits >= 4 && (place == 0 || (shifted && a.n_hits <= INT32_MAX - 4));  // (hits plus 3 in 32 bits)
+  a.win_shift = fits ? place : 0;
+  a.win_whole = fits && (mixed_kernel || !mixed_windows(a)) ? (uint32_t)(a.n_hits - 3) : 0;
+}
+
 // Tracks per work item alone (what the tape's layout depends on).
 inline int32_t item_tracks(int64_t n_tracks, int sms) { return work_shape(n_tracks, 1, 1, sms).tracks; }
 // Clear a launch's counters: the tape's (with the work item counter), the work

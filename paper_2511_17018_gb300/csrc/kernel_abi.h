@@ -119,6 +119,9 @@ struct FitArgs {
   int32_t field;               // field map on (selects the kernel variant that follows it)
   int32_t form;                // factor of the covariance: 0 square root (L), 1 U-D (fast mode without material)
   int32_t item_tracks;         // tracks per work item (1..32, set by the launcher)
+  // windows of 4 clusters, aligned in y (set by the launcher, set_windows in internal.h)
+  int32_t win_shift;           // clusters from the first window's start to cluster 0 (0..3)
+  uint32_t win_whole;          // (uint32_t)h < win_whole: the window that starts at cluster h is copied whole
 };
 
 // Arguments of one backward launch (same frame as the recorded fit).
@@ -196,6 +199,14 @@ constexpr int kFitBlockSmemBytes = 4 * (kTablesFloats + kAlignFloats);
 // phase (rps / 4 + 1 windows) and those of the next one on their way.
 __host__ __device__ constexpr int fit_stage_windows(int rps) { return 2 * (rps / 4) + 1; }
 __host__ __device__ constexpr int fit_warp_stage_bytes(int rps) { return fit_stage_windows(rps) * kWarp * 40; }
+// Whether the fit of a shape stages arrays that begin within a window in windows: all
+// but the shapes for small batches (8 or 16 warps, one block per SM), whose time is
+// their tracks' chains (1,000 tracks, aligned arrays: 158.9 us, with the shift's few
+// instructions 160.9; unaligned ones 185 and 171, and 316 with the copies of single
+// clusters that windows replaced).
+__host__ __device__ constexpr bool fit_shifted(int rps, int warps, int min_blocks) {
+  return !(rps == 4 && warps < 24 && min_blocks == 1);
+}
 // Blocks per SM the fit asks for (__launch_bounds__) at each supported shape.
 __host__ __device__ constexpr int fit_min_blocks(int rps, int warps) { return (rps == 4 && warps == 24) || rps == 16 || warps == 16 ? 1 : 2; }
 

@@ -352,6 +352,8 @@ tpcfit_status rtc_launch_fit(const GeoConst& g, bool det, int rps, int warps, co
   const WorkShape w = work_shape(a.n_tracks, r.blocks, warps, r.sms);
   FitArgs args = a;
   args.item_tracks = w.tracks;
+  // (no variant for arrays without common windows: those are staged cluster by cluster)
+  set_windows(args, false, fit_shifted(rps, warps, fit_min_blocks(rps, warps)));
   if (clear_work(a.work, a.tape != nullptr, needs_work_counter(w), s) != cudaSuccess) return TPCFIT_ECUDA;
   void* params[] = {&args};
   e = cudaLaunchKernel(fn, dim3(w.blocks), dim3(w.warps * kWarp), params,

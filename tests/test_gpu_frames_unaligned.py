@@ -4,8 +4,8 @@ with -m gpu).
 The staging copies clusters in windows of four that reach into the neighbouring
 tracks, so next to a frame's boundary it reads words of the next frame that another
 stream has yet to write; once that frame's flag is set, its own values have to be
-seen.  Arrays shifted by 1 to 3 elements are copied cluster by cluster, aligned ones
-in whole windows."""
+seen.  Arrays that begin at one place within a window are copied in whole windows,
+others cluster by cluster."""
 import numpy as np
 import pytest
 
@@ -20,7 +20,7 @@ FRAMES, TRACKS = 150, 31
 
 
 @pytest.mark.parametrize("lanes", [1, 4])
-@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+@pytest.mark.parametrize("shift", [(0, 0, 0), (1, 1, 1), (3, 3, 3), (1, 2, 3), (0, 0, 1)])
 def test_streamed_frames_at_any_alignment(shift, lanes):
     fr = synth.generate(FRAMES * TRACKS, 71, drop_p=0.05, cap_lengths=True)
     full = tf.frame_to_device(fr)
@@ -32,11 +32,11 @@ def test_streamed_frames_at_any_alignment(shift, lanes):
         ref = {k: v.clone() for k, v in ref.items()}
         assert f.status()[0] == tf.OK
         host, dev = {}, {}
-        for k in ("y", "z", "rowsec"):
+        for k, s in zip(("y", "z", "rowsec"), shift):
             host[k] = full[k].cpu().pin_memory()
             # what is there before: no valid row, clusters far away
-            dev[k] = torch.full((fr.n_hits + shift,), -1 if k == "rowsec" else 1e3, dtype=full[k].dtype,
-                                device="cuda")[shift:]
+            dev[k] = torch.full((fr.n_hits + s,), -1 if k == "rowsec" else 1e3, dtype=full[k].dtype,
+                                device="cuda")[s:]
         batch = FrameBatch(dev["y"], dev["z"], dev["rowsec"], full["offsets"], full["seeds"], base)
         flags = torch.zeros(FRAMES, dtype=torch.int32, device="cuda")
         one = torch.ones(1, dtype=torch.int32).pin_memory()
