@@ -380,20 +380,9 @@ __device__ __forceinline__ void sqrt_from_ud_ckpt(StepState& S) {
 }
 
 // One cluster as stored (y, z, packed row/sector), loaded ahead of its use.
-// A track's clusters and the steps of a pass over it, 0 if it has no fit.  The
-// recording has the last word: of a track without a fit it holds no state and no
-// cluster, whatever the caller's ndf (another fit's, say) makes of it.  The range is
-// empty for the offsets that the fit refuses, so no cluster outside the arrays is
-// touched.
-struct RecordedTrack {
-  int begin = 0, end = 0, steps = 0;
-};
 template <class A>
 __device__ __forceinline__ RecordedTrack recorded_track(const A& a, int32_t trk) {
-  RecordedTrack r;
-  track_range(a.off, trk, a.n_hits, r.begin, r.end);
-  r.steps = a.ndf[trk] > 0 ? min(a.ck_last[trk] + 1, r.end - r.begin) : 0;
-  return r;
+  return tpcfit::recorded_track(a.off, a.n_hits, a.ndf, a.ck_last, trk);
 }
 
 struct HitRaw {
@@ -915,8 +904,8 @@ __device__ __forceinline__ void red_add2(float* p, float v0, float v1) {
 }
 
 // prev: what the inward pass left at cluster h (read ahead by the caller; only
-// the outward pass, pass 0, adds to it).  Clusters that no step of a fitted track
-// reached keep the zeros that the host put there.
+// the outward pass, pass 0, adds to it).  The clusters that no step of a fitted track
+// reaches were cleared before (launch_clear_gradients).
 __device__ __forceinline__ void accumulate_meas_grad(const BwdArgs& a, int pass, int h, int row, int sec, float g0,
                                                      float g1, float2 prev) {
   if (a.grad_meas) {

@@ -18,6 +18,22 @@ __device__ __forceinline__ bool track_range(const int32_t* off, int64_t t, int64
   return false;
 }
 
+// A recorded track's clusters and the steps of a pass over it, 0 if it has no fit.  The
+// recording has the last word: of a track without a fit it holds no state and no
+// cluster, whatever the caller's ndf (another fit's, say) makes of it.  The range is
+// empty for the offsets that the fit refuses, so no cluster outside the arrays is
+// touched.
+struct RecordedTrack {
+  int32_t begin = 0, end = 0, steps = 0;
+};
+__device__ __forceinline__ RecordedTrack recorded_track(const int32_t* off, int64_t n_hits, const int32_t* ndf,
+                                                        const int32_t* ck_last, int64_t t) {
+  RecordedTrack r;
+  track_range(off, t, n_hits, r.begin, r.end);
+  r.steps = ndf[t] > 0 ? min(ck_last[t] + 1, r.end - r.begin) : 0;
+  return r;
+}
+
 // Frame of track `trk`: f with base[f] <= trk < base[f + 1] (base[0] = 0,
 // base[n_frames] = total tracks); -1 if trk lies outside the table.
 __device__ __forceinline__ int frame_of(const int64_t* base, int n_frames, int64_t trk) {

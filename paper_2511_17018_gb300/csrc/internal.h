@@ -118,6 +118,11 @@ cudaError_t smooth_store_det(int64_t& float4s);
 // true if `warps` is a compiled backward block shape
 bool backward_shape_supported(int warps);
 
+// Zero the gradients gm [n_hits][2] (8-byte aligned) of the clusters that the adjoint of
+// a recorded fit does not reach (key_reduce.cu), and the alignment gradient
+// [kAlignFloats] if not null.
+cudaError_t launch_clear_gradients(const int32_t* off, int32_t n_tracks, int64_t n_hits, const int32_t* ndf,
+                                   const int32_t* ck_last, float* gm, float* grad_align, cudaStream_t s);
 // Deterministic per-key reduction of cluster gradients (key_reduce.cu).
 size_t key_sort_scratch_bytes(int64_t n_hits);
 cudaError_t launch_key_sort(const uint16_t* rowsec, int64_t n_hits, int n_rows, void* scratch, int** sorted_out,

@@ -150,12 +150,6 @@ tpcfit_status from_cuda(cudaError_t e) {
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
-// Zero the gradients of all clusters (null: none wanted): the reverse writes those
-// that a step of a fitted track reaches.
-cudaError_t clear_meas_grad(float* gm, int64_t n_hits, cudaStream_t s) {
-  return gm && n_hits > 0 ? cudaMemsetAsync(gm, 0, 2 * sizeof(float) * (size_t)n_hits, s) : cudaSuccess;
-}
-
 // Whether the call's stream is being captured, noted in the handle.
 bool note_capture(tpcfit_handle* h, cudaStream_t s) {
   cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
@@ -661,7 +655,8 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
   cudaStream_t s = (cudaStream_t)stream;
   if (n_tracks == 0) {
     cudaError_t e = cudaMemsetAsync(grad_align, 0, sizeof(float) * kAlignFloats, s);
-    if (e == cudaSuccess) e = clear_meas_grad(grad_meas, hits->n_hits, s);
+    if (e == cudaSuccess && grad_meas && hits->n_hits > 0)
+      e = cudaMemsetAsync(grad_meas, 0, 2 * sizeof(float) * (size_t)hits->n_hits, s);
     return from_cuda(e);
   }
   if (!track_offsets || !ndf || !grad_chi2 || !grad_seeds) return TPCFIT_EINVAL;
@@ -719,8 +714,8 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
     // fast: atomics straight into the alignment gradient
     b.grad_meas = grad_meas;
     b.grad_align_atomic = grad_align;
-    e = cudaMemsetAsync(grad_align, 0, sizeof(float) * kAlignFloats, s);
-    if (e == cudaSuccess) e = clear_meas_grad(grad_meas, hits->n_hits, s);
+    e = grad_meas ? launch_clear_gradients(track_offsets, n_tracks, hits->n_hits, ndf, b.ck_last, grad_meas, grad_align, s)
+                  : cudaMemsetAsync(grad_align, 0, sizeof(float) * kAlignFloats, s);
     if (e == cudaSuccess) e = launch_backward_fast(b, h->bwd_warps, s);
     return from_cuda(e);
   }
@@ -737,9 +732,8 @@ tpcfit_status tpcfit_fit_backward(tpcfit_handle* h, const tpcfit_hits* hits, con
   if (st != TPCFIT_OK) return st;
   b.grad_meas = gm;
   b.grad_align_atomic = nullptr;
-  // the sums below take every cluster, those that no step reaches too (beyond the end
-  // of an outward pass, of no track)
-  e = clear_meas_grad(gm, hits->n_hits, s);
+  // the sums below take every cluster, those that no step reaches too
+  e = launch_clear_gradients(track_offsets, n_tracks, hits->n_hits, ndf, b.ck_last, gm, nullptr, s);
   if (e == cudaSuccess) e = launch_backward_det(b, h->bwd_warps, s);
   if (h->det_reduce == 0) {
     if (e == cudaSuccess)

@@ -123,6 +123,10 @@ cudaError_t backward_store_fast(int, int, int, int64_t& n) { return n = 1 << 20,
 cudaError_t backward_store_det(int, int, int, int64_t& n) { return n = 2 << 20, cudaSuccess; }
 cudaError_t smooth_store_fast(int64_t& n) { return n = 3 << 20, cudaSuccess; }
 cudaError_t smooth_store_det(int64_t& n) { return n = 3 << 20, cudaSuccess; }
+cudaError_t launch_clear_gradients(const int32_t*, int32_t, int64_t, const int32_t*, const int32_t*, float* gm, float*,
+                                   cudaStream_t) {
+  return use(gm), cudaSuccess;
+}
 size_t key_sort_scratch_bytes(int64_t n) { return 16 * (size_t)n; }
 size_t key_fixed_scratch_bytes() { return 131072; }
 cudaError_t launch_key_sort(const uint16_t*, int64_t, int, void* scratch, int**, int**, cudaStream_t) {

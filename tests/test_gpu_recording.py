@@ -116,7 +116,7 @@ def test_offsets_beyond_the_arrays_touch_nothing_outside(kind, where):
         st, code, trk = f.status()
         assert st == tf.EDEVICE and code == 1 and trk in bad
         assert torch.equal(_bits(got["gs"][:, keep]), _bits(want["gs"][:, keep]))
-        assert bool((got["gs"][:, bad] == 0).all())
+        assert bool((got["gs"][:, bad] == 0).all()) and bool((got["gm"][~mine] == 0).all())
         for k in ("gm", "resid", "rcov", "chi2", "state", "state_cov"):
             assert torch.equal(_bits(got[k][mine]), _bits(want[k][mine])), k
         if where == "last":  # in order, but for the arrays' end
