@@ -514,7 +514,7 @@ def main():
         fitter.fit(dev, out)
         mid.record(stream)
 
-    # ---- the step: fit with checkpoints + adjoint
+    # ---- the step: recorded fit + adjoint
     fitter.set_record(True)
     for _ in range(args.warmup):
         fit_adjoint()
@@ -740,7 +740,8 @@ def main():
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "roofline": {"bound": "alu", "achieved": bwd_f["achieved_method"], "peak": peak_tf, "unit": "TFLOP/s",
                      "frac": bwd_f["frac_method"], "traffic": _traffic("backward_" + args.mode),
-                     "kernel": "tape_reverse_ud_kernel", "launch_ms": bwd_ms,
+                     "kernel": "tape_reverse_ud_kernel" if args.mode == "fast" else "tape_reverse_kernel",
+                     "launch_ms": bwd_ms,
                      "frac_impl": bwd_f["frac_impl"], "achieved_impl": bwd_f["achieved_impl"],
                      "count": "achieved/frac: method count (480 flop per cluster for the fit, x2.5 for the reverse); "
                               "*_impl: the form as implemented (flops.py; fast mode: U-D)",
@@ -751,9 +752,11 @@ def main():
                       "traffic": _traffic("fit_" + args.mode)},
         "hits_per_s": value * mhits,
         "e2e": e2e,
-        "gpu_launches": 5 * args.steps,
+        # per step: ordering (2), fit, reverse from the tape, and the reverse from checkpoints of what is not on it
+        # (fast) or the clearing of gradients and the three kernels of the per-key sums (deterministic)
+        "gpu_launches": (5 if args.mode == "fast" else 8) * args.steps,
         "clocks": clocks,
-        "config": {"workload": WORKLOAD, "step": "fit with checkpoints + adjoint (gradients w.r.t. alignment and seeds)",
+        "config": {"workload": WORKLOAD, "step": "recorded fit + adjoint (gradients w.r.t. alignment and seeds)",
                    "mode": args.mode, "tracks": fr.n_tracks, "hits": fr.n_hits, "mean_hits_per_track": mhits,
                    "l2": "inputs larger than L2 (clusters %.0f MB > 126 MB), no flush" % (10 * fr.n_hits / 1e6),
                    "fitted_fraction": float(np.mean(ndf > 0))},

@@ -113,9 +113,11 @@ tpcfit_status tpcfit_set_config(tpcfit_handle* h, int lanes_per_track, int rows_
  * time frame, like the calibration constants of Sec. 4.1. */
 tpcfit_status tpcfit_set_alignment(tpcfit_handle* h, const float* d, void* stream);
 
-/* Pre-size the handle's device scratch for up to max_tracks tracks (the length
- * permutation) so that later fits allocate nothing, e.g. during CUDA-graph
- * capture.  Synchronous. */
+/* Pre-size the length permutation for up to max_tracks tracks, so that later
+ * fits without recording allocate nothing, e.g. during CUDA-graph capture.
+ * max_hits is not used.  Recorded fits, the adjoint, the smoother, the rejection
+ * and batched frames size their own scratch in the first call that needs it: run
+ * one of the same size before a capture.  Synchronous. */
 tpcfit_status tpcfit_reserve(tpcfit_handle* h, int64_t max_tracks, int64_t max_hits);
 
 /* Fit n_tracks tracks.
@@ -230,7 +232,9 @@ const char* tpcfit_rtc_log(void);
  * the free device memory, and in the forms without one (several lanes per track;
  * the fast square-root form without material), the fit leaves checkpoints
  * instead: the state before every 16th step (about 8 floats per cluster, also
- * handle-owned).  Any tpcfit_fit call replaces the recording. */
+ * handle-owned).  The buffers stay with the handle for the next recording; the
+ * tape gives way where a later fit finds no room.  Any tpcfit_fit call replaces
+ * the recording. */
 tpcfit_status tpcfit_set_record(tpcfit_handle* h, int record);
 
 /* Launch configuration of the adjoint's reverse from checkpoints: warps per
@@ -258,7 +262,7 @@ tpcfit_status tpcfit_set_fit_form(tpcfit_handle* h, int form);
  * recomputes its segments in: 1 = U-D (C = U D U^T, U unit upper triangular,
  * Bierman's measurement updates; default), 0 = the square-root factor
  * (C = L L^T, Potter's updates).  Both give the gradient of the same fit; they
- * differ in FP32 rounding and speed (U-D: 15 factor entries instead of 25, 6
+ * differ in FP32 rounding and speed (U-D: 15 factor entries instead of 25, 5
  * float4 per stored state instead of 8).  The square-root reverse needs a
  * recording made in the square-root form (tpcfit_set_fit_form 0, or one lane
  * per track not in effect): its adjoint crosses segment boundaries only if the

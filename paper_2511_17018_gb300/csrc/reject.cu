@@ -1,9 +1,9 @@
 // Outlier rejection after the smoother: every cluster whose leave-one-out
 // chi2 exceeds a cut is dropped from its track, the others are copied in
-// their order.  One warp per track; the kept clusters of 32 consecutive
-// clusters are placed with a ballot and a population count, so the output
-// order is the input order (the cluster-to-track relation the deterministic
-// mode keeps, Sec. 2) and the results do not depend on scheduling.
+// their order.  A warp counts four tracks at once and copies one at a time; the
+// kept clusters of 32 consecutive ones are placed with a ballot and a population
+// count, so the output order is the input order (the cluster-to-track relation the
+// deterministic mode keeps, Sec. 2) and the results do not depend on scheduling.
 //
 // Three kernels: the kept clusters counted; the counts of the blocks' tracks
 // summed up; the clusters copied to where the sums say.  Bound by memory: chi2 is

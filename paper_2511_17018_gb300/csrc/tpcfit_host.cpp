@@ -946,7 +946,7 @@ tpcfit_status tpcfit_fit_adjoint_host(tpcfit_handle* h, const float* y, const fl
   if (e == cudaSuccess) e = cudaMemcpyAsync(b + o_seed, seeds, 20 * N, cudaMemcpyHostToDevice, c);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b + o_g, grad_chi2, 4 * N, cudaMemcpyHostToDevice, c);
   if (e == cudaSuccess) e = cudaEventRecord(h->pipe_in[slot], c);
-  // fit with checkpoints and adjoint on the caller's stream
+  // recorded fit and adjoint on the caller's stream
   if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->pipe_in[slot], 0);
   if (e != cudaSuccess) return from_cuda(e);
   h->pipe_slot = slot ^ 1;
