@@ -1139,8 +1139,8 @@ cudaError_t launch_default(const FitArgs& a, cudaStream_t s) {
     if (warps <= 16) return launch_cfg<4, 16, 1, RECORD, FRAMES, PHYS, FORM>(a, s);
   }
   // arrays without common windows: cluster by cluster, a full batch's staging takes
-  // longer than its arithmetic (400,000 tracks: 1,190 to 1,250 us against 665 aligned,
-  // 700 to 740 so); smaller batches wait for their tracks' chains either way.  (The fast
+  // longer than its arithmetic (400,000 tracks: 1,180 to 1,250 us against 667 aligned,
+  // 680 to 725 so); smaller batches wait for their tracks' chains either way.  (The fast
   // square-root form keeps one kernel: see above.)
   if constexpr (RECORD != 1 && (TPCFIT_DET || FORM == 1))
     if (mixed_windows(a)) return launch_cfg<4, 24, 1, RECORD, FRAMES, PHYS, FORM, true>(a, s);
